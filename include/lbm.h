@@ -53,7 +53,9 @@ extern "C" {
 #define LBM_STORAGE_F16 2    /* stored as FP16 f_i / w_i - rho_ref (FP32 arithmetic) */
 
 #define LBM_KERNEL_AUTO 0    /* the library's choice: with the energy equation on, the two-pass
-                                path for lattices of at most 2^18 nodes, else the fused kernel */
+                                path for lattices of at most 2^18 nodes, else the fused update
+                                by independent warps (one launch per update, two columns per
+                                thread) */
 #define LBM_KERNEL_SPLIT 1   /* density/psi, collide, energy: three launches per update */
 #define LBM_KERNEL_FUSED 2   /* one launch per update; the library picks the columns per thread */
 #define LBM_KERNEL_FUSED_1COL 3 /* the fused kernel with one lattice column per thread */
@@ -104,7 +106,8 @@ typedef struct lbm_info {
   size_t device_bytes;        /* device memory held by the handle */
   int kernel;                 /* kernel path in use (LBM_KERNEL_SPLIT, _FUSED or _TWOPASS) */
   int tile_cols, tile_rows;   /* fused kernel (two-pass path: its first pass): most output
-                                 columns and rows of one CTA's tile (0 on the split path) */
+                                 columns and rows of one CTA's tile (of one warp's, where the
+                                 library's choice sweeps by warps; 0 on the split path) */
   int cols_per_thread;        /* fused kernel: lattice columns each thread sweeps (1 or 2;
                                  0 on the split path) */
 } lbm_info_t;

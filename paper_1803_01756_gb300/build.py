@@ -28,7 +28,8 @@ _FAST = ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]
 # of the 168 that three CTAs per SM allow): GB300, 4096 x 512: 64.9 against 65.1 us per
 # update, FP16 storage 70.5 against 71.2 us; 16384 x 2048: 902.5 against 904.7 us.
 PER_FILE = {"lbm_fused.cu": _FAST + ["-Xptxas=--register-usage-level=8"],
-            "lbm_fused_c2.cu": _FAST, "lbm_fused_batch.cu": _FAST, "lbm_twopass.cu": _FAST}
+            "lbm_fused_c2.cu": _FAST, "lbm_sweep.cu": _FAST,
+            "lbm_sweep_f16.cu": _FAST, "lbm_sweep_bf16.cu": _FAST, "lbm_fused_batch.cu": _FAST, "lbm_twopass.cu": _FAST}
 _lock = threading.Lock()
 
 

@@ -132,6 +132,17 @@ struct DevParams {
   float rho_out;
 };
 
+// Physics constants of the warp sweep (lbm_sweep.cuh), derived from DevParams by
+// sweep_consts: some with their sign turned or summed.
+struct SweepConsts {
+  float rho_ref, b, inv_Tc, xr;
+  float sr, nkappa, kappa1r, ps_g, ps_RT, ps_R, ps_phi, ps_B, ps_3, psi_r2, psi_den;
+  float akap1_cv3, nkappa_r, RTc_cv3, lam23_cv;
+  float G3, G3r;
+  float nk10, k11, k12, k13, k14, k20, k21, k22, k23, k24, kq0, kq1, kq2;
+  float kn0, kn1, kn2, kn3;
+};
+
 // Per-update scalars computed on the host in double precision.
 struct StepScalars {
   float u_in;   // inlet velocity of time t

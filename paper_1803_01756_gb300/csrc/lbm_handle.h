@@ -29,6 +29,7 @@ struct lbm_lattice {
   long long t = 0;
   int kernel = LBM_KERNEL_SPLIT;
   lbm::FusedTiling fused{0, 0, 1};  // CTA tiling of the fused kernel
+  lbm::SweepTiling sweep{0, 0, 0, 0};  // warp sweep (strips = 0: the CTA sweep runs)
   lbm::TwoPassTiling twopass{0, 0};  // row-chunk heights of the two-pass path
   int cur = 0;   // g[cur]: post-collision populations of the previous update
   int tcur = 0;  // T[tcur]: temperature deviation of time t

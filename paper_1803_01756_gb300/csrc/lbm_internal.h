@@ -90,6 +90,30 @@ cudaError_t launch_energy_rk4(const DevParams &p, const float *Tin, float *Tout,
                               const float *ux, const float *uy, unsigned *status,
                               const StepScalars *sc, int Hb, cudaStream_t s);
 
+// warp sweep (lbm_sweep.cu): one launch per update, each warp sweeps a strip of 64 columns
+// through a row chunk on its own
+struct SweepTiling {
+  int strips, chunks;  // warps across the lattice, row chunks
+  int width;           // output columns of a strip
+  int pdl;             // launch each update as a programmatic dependent of the previous one
+};
+// tiling for this device (strips = 0 on failure)
+SweepTiling sweep_tiling(const DevParams &p, int storage, int device);
+cudaError_t launch_sweep(const DevParams &p, int storage, const void *gs, void *gout,
+                         const float *Tin, float *Tout, unsigned *status, const StepScalars *sc,
+                         const SweepTiling &tl, cudaStream_t s);
+
+// the kernels with 16-bit storage (lbm_sweep_f16.cu, lbm_sweep_bf16.cu): resident CTAs per SM
+// and launch
+cudaError_t sweep_f16_occupancy(const DevParams &p, int *occ);
+cudaError_t sweep_f16_launch(const DevParams &p, const void *gs, void *gout, const float *Tin,
+                             float *Tout, unsigned *status, const StepScalars *sc,
+                             const SweepTiling &tl, cudaStream_t s);
+cudaError_t sweep_bf16_occupancy(const DevParams &p, int *occ);
+cudaError_t sweep_bf16_launch(const DevParams &p, const void *gs, void *gout, const float *Tin,
+                              float *Tout, unsigned *status, const StepScalars *sc,
+                              const SweepTiling &tl, cudaStream_t s);
+
 // set-up and reductions
 cudaError_t launch_init(const DevParams &p, int storage, const double *rho0, void *gout,
                         cudaStream_t s);

@@ -1,0 +1,132 @@
+// The single-lattice kernel of the warp sweep (lbm_sweep.cuh) and its launch, templated on the
+// population storage: lbm_sweep.cu (FP32, with the tiling), lbm_sweep_f16.cu and
+// lbm_sweep_bf16.cu instantiate one each, so that the three compile in parallel.
+#pragma once
+#include <algorithm>
+
+#include "lbm_sweep.cuh"
+
+namespace lbm {
+
+namespace {
+
+constexpr int SW = 4;  // warps of a CTA: four adjacent strips, which share their halo columns
+                       // in L1 (one-warp CTAs: 48.4 against 47.9 us on 4096 x 512)
+constexpr int SNT = 32 * SW;
+// Resident CTAs per SM the registers are sized for: 12 warps with 168 registers a thread.
+// Eight warps with 214 registers let the compiler keep more constants but cover less of the
+// latency of a row step (4096 x 512: 52.7 against 48.6 us per update, 16384 x 2048: 664
+// against 575 us, 16-bit storage 987 against 720 us); 16 warps (128 registers) spill.
+constexpr int SMIN = 3;
+
+SweepConsts sweep_consts(const DevParams &p) {
+  SweepConsts k;
+  k.rho_ref = p.rho_ref;
+  k.b = p.eos_b;
+  k.inv_Tc = p.inv_Tc;
+  k.xr = p.xr;
+  k.sr = p.sr;
+  k.nkappa = -p.kappa;
+  k.kappa1r = p.kappa1 + p.rphi_r;
+  k.ps_g = p.ps_g;
+  k.ps_RT = p.ps_RT;
+  k.ps_R = p.ps_R;
+  k.ps_phi = p.ps_phi;
+  k.ps_B = p.ps_B;
+  k.ps_3 = p.ps_3;
+  k.psi_r2 = p.psi_r2;
+  // the denominator psi + psi_r stays positive where both vanish (the quotient is 0 there)
+  k.psi_den = std::max(p.psi_r, 1e-30f);
+  k.akap1_cv3 = p.akap1_cv3;
+  k.nkappa_r = -p.kappa_r;
+  k.RTc_cv3 = p.RTc_cv3;
+  k.lam23_cv = p.lam23_cv;
+  k.G3 = p.G3;
+  k.G3r = p.G3r;
+  k.nk10 = -p.k1[0];
+  k.k11 = p.k1[1];
+  k.k12 = p.k1[2];
+  k.k13 = p.k1[3];
+  k.k14 = p.k1[4];
+  k.k20 = p.k2[0];
+  k.k21 = p.k2[1];
+  k.k22 = p.k2[2];
+  k.k23 = p.k2[3];
+  k.k24 = p.k2[4];
+  k.kq0 = p.kq[0];
+  k.kq1 = p.kq[1];
+  k.kq2 = p.kq[2];
+  k.kn0 = p.kn[0];
+  k.kn1 = p.kn[1];
+  k.kn2 = p.kn[2];
+  k.kn3 = p.kn[3];
+  return k;
+}
+
+template <bool YW, bool XO, bool TH, bool MP, class ST>
+__global__ void __launch_bounds__(SNT, SMIN)
+    k_sweep(const __grid_constant__ DevParams p, const __grid_constant__ SweepConsts k,
+            const typename ST::T *gs, typename ST::T *gout, const float *Tin, float *Tout,
+            unsigned *status, const StepScalars *__restrict__ sc) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const StepScalars ssc = *sc;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int Y0 = (int)(((long long)blockIdx.y * p.ny) / gridDim.y);
+  const int ye = (int)(((long long)(blockIdx.y + 1) * p.ny) / gridDim.y);
+  __shared__ float4 rings[SW][TH ? 4 * 3 * 32 : 32];
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int strip = (int)blockIdx.x * SW + warp;
+  float4 *ring = rings[warp];
+  Sweep<YW, XO, TH, MP, ST> s(p, k, gs, gout, Tin, Tout, ssc, sweep_c0(strip, TH), Y0, ye,
+                              ring);
+  s.run(status);
+}
+
+template <class ST>
+using SweepFn = void (*)(DevParams, SweepConsts, const typename ST::T *, typename ST::T *,
+                         const float *, float *, unsigned *, const StepScalars *);
+
+template <class ST>
+SweepFn<ST> sweep_variant(const DevParams &p) {
+#define KS(a, b, c, d) k_sweep<a, b, c, d, ST>
+  static const SweepFn<ST> table[16] = {
+      KS(false, false, false, false), KS(false, false, false, true), KS(false, false, true, false),
+      KS(false, false, true, true),   KS(false, true, false, false), KS(false, true, false, true),
+      KS(false, true, true, false),   KS(false, true, true, true),   KS(true, false, false, false),
+      KS(true, false, false, true),   KS(true, false, true, false),  KS(true, false, true, true),
+      KS(true, true, false, false),   KS(true, true, false, true),   KS(true, true, true, false),
+      KS(true, true, true, true)};
+#undef KS
+  const int k = (p.y_walls ? 8 : 0) | (p.x_open ? 4 : 0) | (p.thermal ? 2 : 0) |
+                (p.multiphase ? 1 : 0);
+  return table[k];
+}
+
+int sweep_cols(int strips) { return (strips + SW - 1) / SW; }
+
+template <class ST>
+cudaError_t sweep_launch_t(const DevParams &p, const void *gs, void *gout, const float *Tin,
+                           float *Tout, unsigned *status, const StepScalars *sc,
+                           const SweepTiling &tl, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)sweep_cols(tl.strips), (unsigned)tl.chunks);
+  cfg.blockDim = dim3(SNT);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = tl.pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, sweep_variant<ST>(p), p, sweep_consts(p),
+                            static_cast<const typename ST::T *>(gs),
+                            static_cast<typename ST::T *>(gout), Tin, Tout, status, sc);
+}
+
+template <class ST>
+cudaError_t sweep_occupancy_t(const DevParams &p, int *occ) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, sweep_variant<ST>(p), SNT, 0);
+}
+
+}  // namespace
+
+}  // namespace lbm

@@ -345,7 +345,7 @@ def our_arm(args, world, rank, local, dist):
     shares = {k: v[0] / total_ms for k, v in per_kernel.items()}
     top_name = max(shares, key=shares.get)
     top_ms, top_n = per_kernel[top_name]
-    if top_name == "k_fused_step":
+    if top_name in ("k_fused_step", "k_sweep", "k_tile"):
         per_cell = bytes_cell
     elif top_name == "k_stream_collide":
         per_cell = twopass_sc_bytes(4 if args.storage == "f32" else 2)

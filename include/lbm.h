@@ -54,14 +54,14 @@ extern "C" {
 
 #define LBM_KERNEL_AUTO 0    /* the library's choice: with the energy equation on, the two-pass
                                 path for lattices of at most 2^18 nodes, else the fused update
-                                by independent warps (one launch per update, two columns per
-                                thread) */
+                                by rows of warps, one launch per update, two columns per thread */
 #define LBM_KERNEL_SPLIT 1   /* density/psi, collide, energy: three launches per update */
 #define LBM_KERNEL_FUSED 2   /* one launch per update; the library picks the columns per thread */
 #define LBM_KERNEL_FUSED_1COL 3 /* the fused kernel with one lattice column per thread */
 #define LBM_KERNEL_FUSED_2COL 4 /* the fused kernel with two lattice columns per thread */
-#define LBM_KERNEL_TWOPASS 5 /* two launches per update: streaming and collision (Eqs. 6-15),
-                                then the RK4 energy update (Eqs. 16-18) */
+#define LBM_KERNEL_TWOPASS 5 /* streaming and collision (Eqs. 6-15), then the RK4 energy update
+                                (Eqs. 16-18): on lattices of at most 2^18 nodes as the phases
+                                of one launch over tiles, beyond as two launches per update */
 
 /* Problem parameters, copied by value at lbm_create (the caller keeps ownership). */
 typedef struct lbm_params {
@@ -105,11 +105,11 @@ typedef struct lbm_info {
   double T_ref, rho_ref;      /* deviation references of the stored T and populations */
   size_t device_bytes;        /* device memory held by the handle */
   int kernel;                 /* kernel path in use (LBM_KERNEL_SPLIT, _FUSED or _TWOPASS) */
-  int tile_cols, tile_rows;   /* fused kernel (two-pass path: its first pass): most output
-                                 columns and rows of one CTA's tile (of one warp's, where the
-                                 library's choice sweeps by warps; 0 on the split path) */
-  int cols_per_thread;        /* fused kernel: lattice columns each thread sweeps (1 or 2;
-                                 0 on the split path) */
+  int tile_cols, tile_rows;   /* most output columns and rows of one CTA (of one warp, where the
+                                 library's choice sweeps by warps; two-pass path in two
+                                 launches: its first pass; 0 on the split path) */
+  int cols_per_thread;        /* lattice columns each thread works on (1 or 2; 0 on the split
+                                 path) */
 } lbm_info_t;
 
 /* Create a lattice of nx * ny nodes with parameters *p.  Allocates all device
@@ -131,8 +131,9 @@ int lbm_write_fields(lbm_h h, const double *rho, const double *T, void *stream);
    and Zou-He rules, density, pseudopotential (Eqs. 10-11), forces (Eqs. 9, 14, 15),
    velocity (Eq. 13), moment-space collision with Li forcing (Eqs. 6-8) and the RK4
    temperature update (Eqs. 16-18).  Asynchronous: enqueues work on the stream; on the
-   fused path the updates go in chunks of 16, each preceded by a 192-byte copy of its
-   boundary scalars from pinned host memory, and the host may wait for the copy of the
+   fused and two-pass paths the updates go in chunks of 16, each preceded by a 192-byte copy
+   of its boundary scalars from pinned host memory (the kernels of the library's choice take
+   them as launch arguments in a shorter chunk), and the host may wait for the copy of the
    chunk before last.  Calls on different streams must be ordered by the caller (they
    share the lattice state).  LBM_ERR_ARG if the stream is being captured into a CUDA
    graph: each call stages the boundary scalars of its own updates, so a captured call

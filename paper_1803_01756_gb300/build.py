@@ -2,10 +2,10 @@
 
 Each translation unit compiles to an object in parallel, then nvcc links them
 into paper_1803_01756_gb300/_build/liblbm_gb300.so, a plain C ABI shared object
-(include/lbm.h).  The fused-kernel and two-pass units use approximate division and square root
-(about 2 ulp) and flushes denormals to zero (no value of the update comes within
+(include/lbm.h).  The units of the update kernels (PER_FILE) use approximate division and square
+root (about 2 ulp) and flush denormals to zero (no value of the update comes within
 30 orders of magnitude of the denormal range, so only the special-case code of
-the reciprocal and root instructions goes away): its instruction count bounds its
+the reciprocal and root instructions goes away): instruction count bounds their
 speed, and the results are checked against the FP64 oracle like every other path.
 """
 from __future__ import annotations
@@ -27,9 +27,10 @@ _FAST = ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]
 # The single-lattice fused kernel may take more registers for its schedule (156 instead of 150
 # of the 168 that three CTAs per SM allow): GB300, 4096 x 512: 64.9 against 65.1 us per
 # update, FP16 storage 70.5 against 71.2 us; 16384 x 2048: 902.5 against 904.7 us.
-PER_FILE = {"lbm_fused.cu": _FAST + ["-Xptxas=--register-usage-level=8"],
-            "lbm_fused_c2.cu": _FAST, "lbm_sweep.cu": _FAST,
-            "lbm_sweep_f16.cu": _FAST, "lbm_sweep_bf16.cu": _FAST, "lbm_fused_batch.cu": _FAST, "lbm_twopass.cu": _FAST}
+PER_FILE = {"lbm_fused.cu": _FAST + ["-Xptxas=--register-usage-level=8"]}
+PER_FILE.update({f + ".cu": _FAST for f in (
+    "lbm_fused_c2", "lbm_fused_batch", "lbm_twopass", "lbm_sweep", "lbm_sweep_f16",
+    "lbm_sweep_bf16", "lbm_tile", "lbm_tile_f16", "lbm_tile_bf16")})
 _lock = threading.Lock()
 
 

@@ -31,7 +31,7 @@ struct StateHeader {
 
 using namespace lbm_host;
 const char *kKernelNames[KN_COUNT] = {"k_density_psi", "k_collide", "k_energy", "k_fused_step",
-                                       "k_stream_collide", "k_energy_rk4"};
+                                       "k_stream_collide", "k_energy_rk4", "k_sweep", "k_tile"};
 
 
 }  // namespace
@@ -439,19 +439,39 @@ cudaError_t twopass_b(lbm_lattice *h, int k, cudaStream_t s) {
                                 h->status, h->d_sc + k, h->twopass.Hb, s);
 }
 
+// the kernels that take their scalars by value where no graph replays them
+bool scalars_by_value(const lbm_lattice *h) { return h->tile.strips > 0 || h->sweep.strips > 0; }
+
+int fused_kind(const lbm_lattice *h) {
+  return h->tile.strips > 0 ? KN_TILE : h->sweep.strips > 0 ? KN_SWEEP : KN_FUSED;
+}
+
+// the launch of the current update as one kernel (the tile kernel, the warp sweep or the CTA
+// sweep), with the scalars sc in device memory or (sc = nullptr, the first two) val
+cudaError_t one_launch(lbm_lattice *h, const StepScalars *sc, const StepScalars &val,
+                       cudaStream_t s) {
+  const void *gs = h->g[h->cur];
+  void *gout = h->g[1 - h->cur];
+  const float *Tin = h->T[h->tcur];
+  float *Tout = h->T[1 - h->tcur];
+  if (h->tile.strips > 0)
+    return lbm::launch_tile(h->dp, h->p.storage, gs, gout, Tin, Tout, h->status, sc, val, h->tile,
+                            s);
+  if (h->sweep.strips > 0)
+    return lbm::launch_sweep(h->dp, h->p.storage, gs, gout, Tin, Tout, h->status, sc, val,
+                             h->sweep, s);
+  return lbm::launch_fused(h->dp, h->p.storage, gs, gout, Tin, Tout, h->status, sc, h->fused, s);
+}
+
 // the launches of the current update on the fused or the two-pass path, with the scalars
 // of slot k of d_sc
 cudaError_t fused_launch(lbm_lattice *h, int k, cudaStream_t s) {
-  if (h->kernel == LBM_KERNEL_TWOPASS) {
+  if (h->kernel == LBM_KERNEL_TWOPASS && h->tile.strips == 0) {
     cudaError_t e = twopass_a(h, k, s);
     if (e == cudaSuccess && h->dp.thermal) e = twopass_b(h, k, s);
     return e;
   }
-  if (h->sweep.strips > 0)
-    return lbm::launch_sweep(h->dp, h->p.storage, h->g[h->cur], h->g[1 - h->cur], h->T[h->tcur],
-                             h->T[1 - h->tcur], h->status, h->d_sc + k, h->sweep, s);
-  return lbm::launch_fused(h->dp, h->p.storage, h->g[h->cur], h->g[1 - h->cur], h->T[h->tcur],
-                           h->T[1 - h->tcur], h->status, h->d_sc + k, h->fused, s);
+  return one_launch(h, h->d_sc + k, StepScalars{}, s);
 }
 
 // Scalars of updates t .. t + m - 1 into d_sc, through the staging buffer whose previous
@@ -510,9 +530,11 @@ int fused_steps(lbm_lattice *h, long nsteps, cudaStream_t s) {
   const int C = lbm_lattice::kChunk;
   for (long done = 0; done < nsteps;) {
     const int m = (int)std::min<long>(C, nsteps - done);
-    int rc = stage_scalars(h, m, s);
+    const bool graph = m == C && h->use_graph && !h->timing;
+    const bool value = !graph && scalars_by_value(h);
+    int rc = value ? LBM_OK : stage_scalars(h, m, s);
     if (rc) return rc;
-    if (m == C && h->use_graph && !h->timing) {
+    if (graph) {
       if (!h->gexec[h->cur][h->tcur]) {
         rc = capture_chunk(h);
         if (rc) return rc;
@@ -521,7 +543,10 @@ int fused_steps(lbm_lattice *h, long nsteps, cudaStream_t s) {
       h->t += C;  // an even chunk ends at the parity it started from
     } else {
       for (int k = 0; k < m; k++) {
-        if (h->kernel == LBM_KERNEL_TWOPASS) {
+        if (value) {
+          const StepScalars sc = scalars_at(h, h->t);
+          rc = timed(h, fused_kind(h), s, [&] { return one_launch(h, nullptr, sc, s); });
+        } else if (h->kernel == LBM_KERNEL_TWOPASS) {
           rc = timed(h, KN_STREAM_COLLIDE, s, [&] { return twopass_a(h, k, s); });
           if (!rc && h->dp.thermal)
             rc = timed(h, KN_ENERGY_RK4, s, [&] { return twopass_b(h, k, s); });
@@ -674,18 +699,27 @@ int lbm_create(int nx, int ny, const lbm_params_t *p, lbm_h *out) {
   if (p->x_bc == LBM_X_PRESSURE_INLET)
     h->rho_branch_end = vapour_branch_end(*p, h->Tc, h->Tc * p->T_inlet);
   h->kernel = LBM_KERNEL_SPLIT;
-  // The library's choice for the energy equation on lattices of at most 2^18 nodes is the
-  // two-pass path: its halos are one row (collision) and four rows (energy update) where
-  // the fused kernel's short row chunks on a small lattice spend most row steps filling
-  // its six-stage pipeline (GB300: 200 x 50 9.6 against 11.1 us per update, 1024 x 256
-  // 18.9 against 19.7 us; from 2048 x 256 on the fused kernel is faster).
-  const bool auto_two = p->kernel == LBM_KERNEL_AUTO && p->thermal &&
-                        (long long)nx * ny <= (1LL << 18) && lbm::fused_supported(h->dp);
-  if (auto_two) {
-    h->twopass = lbm::twopass_tiling(h->dp, p->storage, h->device);
-    if (h->twopass.Ha > 0) h->kernel = LBM_KERNEL_TWOPASS;
+  // Lattices of at most 2^18 nodes take the tile kernel, where the two-pass path and the
+  // library's choice meet: all rows of a tile at once instead of a pipeline along the rows
+  // (GB300, us per update, two-pass kernels / tile kernel: 200 x 50 9.6 / 3.6, 1600 x 48 13.9 /
+  // 4.3, 1024 x 128 14.7 / 6.7, 777 x 333 18.9 / 11.7, where the warp sweep takes 17.4;
+  // 2048 x 256 28.1 / 21.6, and 21.3 with the warp sweep, which is ahead beyond).
+  const bool small = (long long)nx * ny <= (1LL << 18) && lbm::fused_supported(h->dp);
+  if (small && ((p->kernel == LBM_KERNEL_AUTO) || p->kernel == LBM_KERNEL_TWOPASS)) {
+    int height = 0;
+    // LBM_TWOPASS_TILE="Ha,Hb" sets the rows per CTA to Ha (tuning experiments)
+    if (const char *env = p->kernel == LBM_KERNEL_TWOPASS ? std::getenv("LBM_TWOPASS_TILE") : nullptr) {
+      int Ha = 0, Hb = 0;
+      if (std::sscanf(env, "%d,%d", &Ha, &Hb) == 2 && Ha >= 1 && Hb >= 1) height = Ha;
+    }
+    h->tile = lbm::tile_tiling(h->dp, p->storage, h->device, height);
+    if (h->tile.strips > 0)
+      h->kernel = p->kernel == LBM_KERNEL_TWOPASS || p->thermal ? LBM_KERNEL_TWOPASS
+                                                                : LBM_KERNEL_FUSED;
   }
-  if (p->kernel == LBM_KERNEL_TWOPASS) {
+  if (h->tile.strips > 0) {
+    // chosen above
+  } else if (p->kernel == LBM_KERNEL_TWOPASS) {
     // 32-bit element offsets, as on the fused path
     if (lbm::fused_supported(h->dp)) h->twopass = lbm::twopass_tiling(h->dp, p->storage, h->device);
     // LBM_TWOPASS_TILE="Ha,Hb" overrides the row-chunk heights (tuning experiments)
@@ -700,14 +734,13 @@ int lbm_create(int nx, int ny, const lbm_params_t *p, lbm_h *out) {
       return LBM_ERR_ARG;
     }
     h->kernel = LBM_KERNEL_TWOPASS;
-  } else if (p->kernel == LBM_KERNEL_AUTO && h->kernel != LBM_KERNEL_TWOPASS &&
-             lbm::fused_supported(h->dp) &&
+  } else if (p->kernel == LBM_KERNEL_AUTO && lbm::fused_supported(h->dp) &&
              // the library's choice of fused kernel: independent warps (64.6 -> 47.9 us per
              // update on 4096 x 512, 902 -> 561 us on 16384 x 2048; 16-bit storage 70.3 ->
              // 54.0 us)
              (h->sweep = lbm::sweep_tiling(h->dp, p->storage, h->device)).strips > 0) {
     h->kernel = LBM_KERNEL_FUSED;
-  } else if (p->kernel != LBM_KERNEL_SPLIT && h->kernel != LBM_KERNEL_TWOPASS) {
+  } else if (p->kernel != LBM_KERNEL_SPLIT) {
     // lattice columns per thread of the fused kernel: as asked, else the library's
     // default, which LBM_FUSED_CPT=1|2 overrides (tuning experiments)
     int cpt = default_cpt(nx, ny);
@@ -951,11 +984,19 @@ int lbm_info(lbm_h h, lbm_info_t *info) {
   info->kernel = h->kernel;
   const bool fused = h->kernel == LBM_KERNEL_FUSED;
   const bool two = h->kernel == LBM_KERNEL_TWOPASS;
-  const bool sweep = fused && h->sweep.strips > 0;
-  info->tile_cols = sweep ? h->sweep.width : fused ? h->fused.W : two ? lbm::twopass_width_a() : 0;
-  info->tile_rows = sweep ? (h->ny + h->sweep.chunks - 1) / h->sweep.chunks
-                    : fused ? h->fused.H : two ? h->twopass.Ha : 0;
-  info->cols_per_thread = sweep ? 2 : fused ? h->fused.cpt : two ? 1 : 0;
+  if (h->tile.strips > 0) {
+    info->tile_cols = h->tile.width;
+    info->tile_rows = h->tile.height;
+    info->cols_per_thread = 2;
+  } else if (h->sweep.strips > 0) {
+    info->tile_cols = h->sweep.width;
+    info->tile_rows = (h->ny + h->sweep.chunks - 1) / h->sweep.chunks;
+    info->cols_per_thread = 2;
+  } else {
+    info->tile_cols = fused ? h->fused.W : two ? lbm::twopass_width_a() : 0;
+    info->tile_rows = fused ? h->fused.H : two ? h->twopass.Ha : 0;
+    info->cols_per_thread = fused ? h->fused.cpt : two ? 1 : 0;
+  }
   return LBM_OK;
 }
 

@@ -9,7 +9,10 @@
 
 namespace lbm_host {
 
-enum { KN_DENSITY = 0, KN_COLLIDE, KN_ENERGY, KN_FUSED, KN_STREAM_COLLIDE, KN_ENERGY_RK4, KN_COUNT };
+enum {
+  KN_DENSITY = 0, KN_COLLIDE, KN_ENERGY, KN_FUSED, KN_STREAM_COLLIDE, KN_ENERGY_RK4, KN_SWEEP,
+  KN_TILE, KN_COUNT
+};
 
 struct TimedLaunch {
   int kind;
@@ -30,6 +33,7 @@ struct lbm_lattice {
   int kernel = LBM_KERNEL_SPLIT;
   lbm::FusedTiling fused{0, 0, 1};  // CTA tiling of the fused kernel
   lbm::SweepTiling sweep{0, 0, 0, 0};  // warp sweep (strips = 0: the CTA sweep runs)
+  lbm::TileTiling tile{0, 0, 0, 0, 0};  // tile kernel (strips = 0: another kernel runs)
   lbm::TwoPassTiling twopass{0, 0};  // row-chunk heights of the two-pass path
   int cur = 0;   // g[cur]: post-collision populations of the previous update
   int tcur = 0;  // T[tcur]: temperature deviation of time t

@@ -91,7 +91,7 @@ cudaError_t launch_energy_rk4(const DevParams &p, const float *Tin, float *Tout,
                               const StepScalars *sc, int Hb, cudaStream_t s);
 
 // warp sweep (lbm_sweep.cu): one launch per update, each warp sweeps a strip of 64 columns
-// through a row chunk on its own
+// through a row chunk on its own; sc as for launch_tile
 struct SweepTiling {
   int strips, chunks;  // warps across the lattice, row chunks
   int width;           // output columns of a strip
@@ -101,18 +101,43 @@ struct SweepTiling {
 SweepTiling sweep_tiling(const DevParams &p, int storage, int device);
 cudaError_t launch_sweep(const DevParams &p, int storage, const void *gs, void *gout,
                          const float *Tin, float *Tout, unsigned *status, const StepScalars *sc,
-                         const SweepTiling &tl, cudaStream_t s);
+                         const StepScalars &val, const SweepTiling &tl, cudaStream_t s);
 
 // the kernels with 16-bit storage (lbm_sweep_f16.cu, lbm_sweep_bf16.cu): resident CTAs per SM
 // and launch
 cudaError_t sweep_f16_occupancy(const DevParams &p, int *occ);
 cudaError_t sweep_f16_launch(const DevParams &p, const void *gs, void *gout, const float *Tin,
                              float *Tout, unsigned *status, const StepScalars *sc,
-                             const SweepTiling &tl, cudaStream_t s);
+                             const StepScalars &val, const SweepTiling &tl, cudaStream_t s);
 cudaError_t sweep_bf16_occupancy(const DevParams &p, int *occ);
 cudaError_t sweep_bf16_launch(const DevParams &p, const void *gs, void *gout, const float *Tin,
                               float *Tout, unsigned *status, const StepScalars *sc,
-                              const SweepTiling &tl, cudaStream_t s);
+                              const StepScalars &val, const SweepTiling &tl, cudaStream_t s);
+
+// tile kernel (lbm_tile.cu): one launch per update, a CTA per strip of 64 columns and row
+// chunk, with a warp for every row of a tile and its halo
+struct TileTiling {
+  int strips, chunks;  // CTAs across and along the lattice (strips = 0: none)
+  int rows;            // most output rows of a tile
+  int width;           // output columns of a strip
+  int height;          // most rows of a CTA, swept tile by tile
+};
+// tiling for this device: the library's choice, or `height` rows per CTA when positive
+TileTiling tile_tiling(const DevParams &p, int storage, int device, int height);
+int tile_max_rows(bool thermal);
+// sc: the update's scalars in device memory, or nullptr to pass them by value
+cudaError_t launch_tile(const DevParams &p, int storage, const void *gs, void *gout,
+                        const float *Tin, float *Tout, unsigned *status, const StepScalars *sc,
+                        const StepScalars &val, const TileTiling &tl, cudaStream_t s);
+// the kernels with 16-bit storage (lbm_tile_f16.cu, lbm_tile_bf16.cu)
+cudaError_t tile_f16_occupancy(const DevParams &p, int rows, int *occ);
+cudaError_t tile_f16_launch(const DevParams &p, const void *gs, void *gout, const float *Tin,
+                            float *Tout, unsigned *status, const StepScalars *sc,
+                            const StepScalars &val, const TileTiling &tl, cudaStream_t s);
+cudaError_t tile_bf16_occupancy(const DevParams &p, int rows, int *occ);
+cudaError_t tile_bf16_launch(const DevParams &p, const void *gs, void *gout, const float *Tin,
+                             float *Tout, unsigned *status, const StepScalars *sc,
+                             const StepScalars &val, const TileTiling &tl, cudaStream_t s);
 
 // set-up and reductions
 cudaError_t launch_init(const DevParams &p, int storage, const double *rho0, void *gout,

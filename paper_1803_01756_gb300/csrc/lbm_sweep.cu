@@ -41,14 +41,14 @@ SweepTiling sweep_tiling(const DevParams &p, int storage, int device) {
 
 cudaError_t launch_sweep(const DevParams &p, int storage, const void *gs, void *gout,
                          const float *Tin, float *Tout, unsigned *status, const StepScalars *sc,
-                         const SweepTiling &tl, cudaStream_t s) {
+                         const StepScalars &val, const SweepTiling &tl, cudaStream_t s) {
   switch (storage) {
     case STORAGE_BF16:
-      return sweep_bf16_launch(p, gs, gout, Tin, Tout, status, sc, tl, s);
+      return sweep_bf16_launch(p, gs, gout, Tin, Tout, status, sc, val, tl, s);
     case STORAGE_F16:
-      return sweep_f16_launch(p, gs, gout, Tin, Tout, status, sc, tl, s);
+      return sweep_f16_launch(p, gs, gout, Tin, Tout, status, sc, val, tl, s);
     default:
-      return sweep_launch_t<StoreF32>(p, gs, gout, Tin, Tout, status, sc, tl, s);
+      return sweep_launch_t<StoreF32>(p, gs, gout, Tin, Tout, status, sc, val, tl, s);
   }
 }
 

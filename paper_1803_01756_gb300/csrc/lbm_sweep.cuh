@@ -12,183 +12,31 @@
 //                (Eqs. 6-8) and the store of the populations
 //   S2 row r-2 : div u and the first RK4 slope h1 of Eq. 16 (Eq. 18)
 //   S3 row r-3 : h2      S4 row r-4 : h3      S5 row r-5 : h4 and Eq. 17
-// The 9-point stencils are separable: with s = c + (up + down)/4 and d = up - down of a
-// column's three rows,
-//   g_x = s_E - s_W,   g_y = d + (d_E + d_W)/4,   L = s_E + s_W + (up + down) - 5 c
-// are the gradient and Laplacian sums of rk_rate (lbm_fused_tile.cuh), so a stage takes four
-// shuffles for its two columns instead of nine shared-memory reads for one.  The two
-// columns of a lane are the two lanes of the packed FP32 instructions: every operation of a
-// node that is not an approximate reciprocal or root is half an instruction.
-//
-// With the energy equation the outer 5 columns on each side are halo (54 of 64 columns are
-// outputs) and 5 rows below and above the chunk are swept too; without it one row, and one
-// pair of columns (60 outputs).  Halo nodes are recomputed by the same instructions, so a
-// node has the same bits whichever warp and column slot own it.
+// The lane's arithmetic is in lbm_lane.cuh.  With the energy equation 5 rows below and above
+// the chunk are swept too, without it one.
 #pragma once
 
-#include "lbm_internal.h"
+#include "lbm_lane.cuh"
 
 namespace lbm {
 
 namespace {
 
-using V = float2;  // the values of a lane's two columns
-
-__device__ __forceinline__ V vset(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ V vdup(float a) { return make_float2(a, a); }
-__device__ __forceinline__ V operator+(V a, V b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ V operator*(V a, V b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ V vfma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
-// a - b as (-1) b + a: rounds once, like the subtraction
-__device__ __forceinline__ V operator-(V a, V b) { return __ffma2_rn(vdup(-1.0f), b, a); }
-__device__ __forceinline__ float rcp_approx(float a) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return r;
-}
-__device__ __forceinline__ V vrcp(V a) { return vset(rcp_approx(a.x), rcp_approx(a.y)); }
-// a copy through the packed adder: one instruction for the pair instead of two moves
-__device__ __forceinline__ V vcopy(V a) {
-  return __fadd2_rn(a, make_float2(0.0f, 0.0f));
-}
-__device__ __forceinline__ V vsqrt(V a) { return vset(sqrtf(a.x), sqrtf(a.y)); }
-__device__ __forceinline__ V vrsqrt(V a) { return vset(rsqrtf(a.x), rsqrtf(a.y)); }
-
-// A constant operand.  The two-lane instructions take it as a register pair that holds it
-// twice (PACK), which pays for constants used several times a step; one used once costs more
-// instructions to put into a pair than two scalar operations with the constant as an
-// immediate or from the constant bank (4096 x 512: 48.6 us per update with this split, 50.6
-// with every constant in a pair; 16384 x 2048: 575 and 617 us).
-template <bool PACK>
-struct KC {
-  float v;
-};
-using KL = KC<true>;   // literal
-using KP = KC<true>;   // parameter used several times a step
-using K1 = KC<false>;  // parameter or literal used once a step
-template <bool PK>
-__device__ __forceinline__ V operator*(KC<PK> c, V a) {
-  return PK ? __fmul2_rn(vdup(c.v), a) : vset(c.v * a.x, c.v * a.y);
-}
-template <bool PK>
-__device__ __forceinline__ V operator+(KC<PK> c, V a) {
-  return PK ? __fadd2_rn(vdup(c.v), a) : vset(c.v + a.x, c.v + a.y);
-}
-template <bool PK>
-__device__ __forceinline__ V vfma(KC<PK> c, V a, V b) {
-  return PK ? __ffma2_rn(vdup(c.v), a, b) : vset(fmaf(c.v, a.x, b.x), fmaf(c.v, a.y, b.y));
-}
-// a c + k with a constant addend
-template <bool PK>
-__device__ __forceinline__ V vfma(V a, V b, KC<PK> c) {
-  return PK ? __ffma2_rn(a, b, vdup(c.v)) : vset(fmaf(a.x, b.x, c.v), fmaf(a.y, b.y, c.v));
-}
-template <bool PA, bool PB>
-__device__ __forceinline__ V vfma(KC<PA> c, V a, KC<PB> d) {
-  return PA && PB ? __ffma2_rn(vdup(c.v), a, vdup(d.v))
-                  : vset(fmaf(c.v, a.x, d.v), fmaf(c.v, a.y, d.v));
-}
-// c - a
-template <bool PK>
-__device__ __forceinline__ V operator-(KC<PK> c, V a) {
-  return PK ? vdup(c.v) - a : vset(c.v - a.x, c.v - a.y);
-}
-__device__ __forceinline__ KL kl(float v) { return KL{v}; }
-__device__ __forceinline__ KP kp(float v) { return KP{v}; }
-__device__ __forceinline__ K1 k1(float v) { return K1{v}; }
-
-constexpr unsigned kAll = 0xffffffffu;
-
-__device__ __forceinline__ int modi(int v, int n) {
-  v %= n;
-  return v < 0 ? v + n : v;
-}
-
-// columns of halo on each side of a warp's outputs, and its output columns
-__host__ __device__ constexpr int sweep_halo(bool th) { return th ? 5 : 2; }
-__host__ __device__ constexpr int sweep_width(bool th) { return 64 - 2 * sweep_halo(th); }
-// rows of halo below and above a chunk
-__host__ __device__ constexpr int sweep_rows(bool th) { return th ? 5 : 1; }
-// first even column of strip k (outputs [c + halo, c + halo + width), clipped to the
-// lattice)
-__host__ __device__ constexpr int sweep_c0(int k, bool th) {
-  return k * sweep_width(th) - (th ? 6 : 2);
-}
-__host__ __device__ constexpr int sweep_strips(int nx, bool th) {
-  return (nx + (th ? 1 : 0) + sweep_width(th) - 1) / sweep_width(th);
-}
-
-// Loads of one population and of an aligned column pair, converted as the storage's load
-// does.  Plain (coherent) loads: the kernel may start while the previous update still runs,
-// and a read-only load could be moved above its wait for that update.
-template <class ST>
-__device__ __forceinline__ float pop(const typename ST::T *p, int i);
-template <>
-__device__ __forceinline__ float pop<StoreF32>(const float *p, int) { return *p; }
-template <>
-__device__ __forceinline__ float pop<StoreBF16>(const __nv_bfloat16 *p, int i) {
-  return wlat(i) * __bfloat162float(*p);
-}
-template <>
-__device__ __forceinline__ float pop<StoreF16>(const __half *p, int i) {
-  return wlat(i) * __half2float(*p);
-}
-template <class ST>
-__device__ __forceinline__ V pop2(const typename ST::T *p, int i);
-template <>
-__device__ __forceinline__ V pop2<StoreF32>(const float *p, int) {
-  return *reinterpret_cast<const float2 *>(p);
-}
-template <>
-__device__ __forceinline__ V pop2<StoreBF16>(const __nv_bfloat16 *p, int i) {
-  const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
-  return vset(wlat(i) * v.x, wlat(i) * v.y);
-}
-template <>
-__device__ __forceinline__ V pop2<StoreF16>(const __half *p, int i) {
-  const float2 v = __half22float2(*reinterpret_cast<const __half2 *>(p));
-  return vset(wlat(i) * v.x, wlat(i) * v.y);
-}
-
 // One warp's sweep: the strip with first column C0, output rows [Y0, ye).
 template <bool YW, bool XO, bool TH, bool MP, class ST>
-struct Sweep {
-  using T = typename ST::T;
-  static constexpr int HR = sweep_rows(TH);  // halo rows
-  static constexpr int HC = sweep_halo(TH);  // halo columns
-  static constexpr unsigned E = sizeof(T);
+struct Sweep : Lane<YW, XO, TH, MP, ST> {
+  using L = Lane<YW, XO, TH, MP, ST>;
+  using typename L::Own;
+  using typename L::T;
+  using L::g, L::Tn, L::p, L::k, L::c0, L::sc, L::e_in, L::e_out, L::ends;
+  static constexpr int HR = L::HR;
   static constexpr int NW = HR > 2 ? HR : 2;  // lowest row r whose step reaches no wall below
 
-  const DevParams &p;
-  const SweepConsts &k;
-  const T *gs;
-  T *gout;
-  const float *Tin;
-  float *Tout;
-  const StepScalars &sc;
   int Y0, ye;
-  // Geometry of the lane: its first column c0 (even), the lattice column x0 it loads from
-  // (c0 wrapped into a periodic lattice, clamped beyond an open end, where the loaded
-  // values are replaced or never used), and element offsets from x0 to the second column
-  // (o1), the west source of the first (oW) and the east source of the second (oE).
-  int c0, x0, o1, oW, oE;
-  bool vec;            // the column pair is one aligned pair of elements
-  bool e_in, e_out, ends;  // the warp holds the inlet (outlet) column or its ghost; either
-  bool has_g, tau_const;
-  float in_u;          // velocity inlet: U / (1 - U)
-  unsigned span;       // rows NW .. NW + span - 1 are away from the walls
-  bool outp;           // the lane stores its pair's populations
-  bool out_x, out_y;   // the first (second) column is column nx - 1
-  bool oddx;           // the second column of the pair lies beyond the lattice
-  bool out0, out1;     // output columns
-
-  struct Own {  // values of a node that its RK4 stages share
-    V nux, nuy, cl, Tb, nE1, nE2;
-  };
+  unsigned span;          // rows NW .. NW + span - 1 are away from the walls
   // Carried from row step to row step; an array of two is indexed by the parity of the
   // row's step, so that with two steps per loop iteration few values are copied.
-  V g[9], Tn;             // populations and temperature of the next row, in flight
-  V m[2][9];              // moments of a row: drho, -n1, n2, jx, n4, jy, n6, n7, n8
+  V m[2][9];              // moments of a row
   V psi[2];               // psi - psi_r
   V cfx[2], cfz[2], cl;   // energy coefficients
   V ux[2], uy[2];
@@ -196,232 +44,32 @@ struct Sweep {
   V K2[2], K3[2], K4[2];  // RK stage fields
   V acc1, acc2, acc3;     // sums h1, h1 + 2 h2, h1 + 2 h2 + 2 h3 of three rows
   float4 *own_s;          // the lane's slots in the warp's ring of four rows: [row][3][32]
-  unsigned st;
-  float drho_min, drho_max, dT_min;
-  V chk;                  // not finite once a stored value is not
 
   __device__ __forceinline__ Sweep(const DevParams &p_, const SweepConsts &k_, const T *gs_,
                                    T *gout_, const float *Tin_, float *Tout_,
                                    const StepScalars &sc_, int C0, int Y0_, int ye_,
                                    float4 *ring)
-      : p(p_), k(k_), gs(gs_), gout(gout_), Tin(Tin_), Tout(Tout_), sc(sc_), Y0(Y0_), ye(ye_) {
-    const int lane = (int)(threadIdx.x & 31);
-    own_s = ring + lane;
-    c0 = C0 + 2 * lane;
-    o1 = 1;
-    oW = -1;
-    oE = 2;
-    if (XO) {
-      x0 = min(max(c0, 0), (p.nx - 1) & ~1);
-      vec = true;
-    } else {
-      x0 = modi(c0, p.nx);
-      o1 = modi(c0 + 1, p.nx) - x0;
-      oW = modi(c0 - 1, p.nx) - x0;
-      oE = modi(c0 + 2, p.nx) - x0;
-      vec = (p.nx & 1) == 0;
-    }
+      : L(p_, k_, gs_, gout_, Tin_, Tout_, sc_, C0), Y0(Y0_), ye(ye_) {
+    own_s = ring + (threadIdx.x & 31);
     span = (unsigned)max(0, p.ny - 2 - NW);
-    in_u = XO ? sc.u_in / (1.0f - sc.u_in) : 0.0f;
-    has_g = p.has_g;
-    tau_const = p.tau_const;
-    e_in = XO && C0 <= 0;
-    e_out = XO && C0 + 63 >= p.nx - 1;
-    ends = e_in || e_out;
-    out_x = XO && c0 == p.nx - 1;
-    out_y = XO && c0 + 1 == p.nx - 1;
-    const bool in0 = c0 >= 0 && c0 < p.nx, in1 = c0 + 1 >= 0 && c0 + 1 < p.nx;
-    outp = lane >= HC / 2 && lane < 32 - HC / 2 && in0;
-    oddx = !in1;
-    out0 = 2 * lane >= HC && 2 * lane < 64 - HC && in0;
-    out1 = 2 * lane + 1 >= HC && 2 * lane + 1 < 64 - HC && in1;
     const V z = vdup(0.0f);
 #pragma unroll
-    for (int i = 0; i < 9; i++) g[i] = m[0][i] = m[1][i] = z;
+    for (int i = 0; i < 9; i++) m[0][i] = m[1][i] = z;
 #pragma unroll
     for (int i = 0; i < 2; i++)
       psi[i] = cfx[i] = cfz[i] = ux[i] = uy[i] = K2[i] = K3[i] = K4[i] = z;
-    Tn = cl = T1 = T2 = T3 = acc1 = acc2 = acc3 = chk = z;
-    st = 0u;
-    drho_min = drho_max = dT_min = 0.0f;
+    cl = T1 = T2 = T3 = acc1 = acc2 = acc3 = z;
   }
 
-  // ---- neighbour columns and open ends ----
-  // West neighbour of the first column and east neighbour of the second, from the lanes
-  // beside.  Ghost columns beyond an open end (fix: some warps of the strip only): the outlet
-  // ghost, column nx, copies column nx - 1, so that column is its own east neighbour; the
-  // inlet ghost, column -1, is either a column of its own values or (copy_in) copies column 0.
-  __device__ __forceinline__ void neighbours(V &a, bool copy_in, float &w, float &e) const {
-    if (XO && ends && out_x) a.y = a.x;
-    w = __shfl_up_sync(kAll, a.y, 1);
-    e = __shfl_down_sync(kAll, a.x, 1);
-    if (XO && ends) {
-      if (out_y) e = a.y;
-      if (copy_in && c0 == 0) w = a.x;
-    }
-  }
-  // Separable sums of a 9-point stencil (see the file comment): g_x, g_y and, for the
-  // Laplacian, s_E + s_W and up + down.  (The neighbours inside the pair are the lane's own
-  // registers: scalar operations take them as they are, a packed one would first copy them
-  // into a register pair.)
-  struct Sten {
-    V gx, gy, es, a;
-  };
-  __device__ __forceinline__ Sten stencil(V dn, V c, V up, bool copy_in) const {
-    Sten r;
-    r.a = up + dn;
-    const KL q = kl(0.25f);
-    V s = vfma(q, r.a, c), d = up - dn;
-    float w, e, dw, de;
-    neighbours2(s, d, copy_in, w, e, dw, de);
-    r.gx = vset(s.y - w, e - s.x);
-    r.es = vset(s.y + w, e + s.x);
-    r.gy = vfma(q, vset(d.y + dw, de + d.x), d);
-    return r;
-  }
-  __device__ __forceinline__ void neighbours2(V &s, V &d, bool copy_in, float &w, float &e,
-                                              float &dw, float &de) const {
-    if (XO && ends) {
-      neighbours(s, copy_in, w, e);
-      neighbours(d, copy_in, dw, de);
-    } else {
-      w = __shfl_up_sync(kAll, s.y, 1);
-      e = __shfl_down_sync(kAll, s.x, 1);
-      dw = __shfl_up_sync(kAll, d.y, 1);
-      de = __shfl_down_sync(kAll, d.x, 1);
-    }
-  }
-
-  __device__ __forceinline__ bool ghost(int j) const {
-    return XO && (c0 + j < 0 || c0 + j >= p.nx);
-  }
-  // the inlet ghost, column -1, is the second column of the lane with c0 = -2
-  __device__ __forceinline__ V inlet_set(V a, float v) const {
-    if (c0 == -2) a.y = v;
-    return a;
-  }
-  // Zou-He on the boundary columns of row r (see pull_fix): every lane computes the rule on
-  // its own column, the boundary column's lane keeps the result
-  __device__ __forceinline__ void inlet_fix(int r) {
-    const float known = g[0].x + g[2].x + g[4].x + 2.0f * (g[3].x + g[6].x + g[7].x);
-    // momentum rho U of the end: the pressure inlet gives rho, U = 1 - (known + rho_ref) / rho;
-    // the velocity inlet gives U, rho = (known + rho_ref) / (1 - U) (in_u = U / (1 - U))
-    const float m = p.p_inlet ? sc.rho_in - p.rho_ref - known : (known + p.rho_ref) * in_u;
-    const float g1 = fmaf(2.0f / 3.0f, m, g[3].x);
-    const float d24 = 0.5f * (g[2].x - g[4].x), m6 = m * (1.0f / 6.0f);
-    const float g5 = (g[7].x - d24) + m6, g8 = (g[6].x + d24) + m6;
-    const bool me = c0 == 0;
-    if (me) g[1].x = g1;
-    if (me && !(YW && r == 0)) g[5].x = g5;  // the link from below is a fluid one
-    if (me && !(YW && r == p.ny - 1)) g[8].x = g8;
-  }
-  __device__ __forceinline__ void outlet_rule(const float (&f)[9], float &f3, float &f6,
-                                              float &f7) const {
-    // momentum rho U of the end
-    const float m = f[0] + f[2] + f[4] + 2.0f * (f[1] + f[5] + f[8]) + (p.rho_ref - p.rho_out);
-    const float d24 = 0.5f * (f[2] - f[4]), m6 = m * (1.0f / 6.0f);
-    f3 = fmaf(-2.0f / 3.0f, m, f[1]);
-    f7 = (f[5] + d24) - m6;
-    f6 = (f[8] - d24) - m6;
-  }
-  __device__ __forceinline__ void outlet_fix(int r) {
-    const bool lo = YW && r == 0, hi = YW && r == p.ny - 1, odd = (p.nx & 1) != 0;
-    float f[9], f3, f6, f7;
-#pragma unroll
-    for (int i = 0; i < 9; i++) f[i] = odd ? g[i].x : g[i].y;
-    outlet_rule(f, f3, f6, f7);
-    const bool mx = out_x, my = out_y;
-    if (mx) g[3].x = f3;
-    if (my) g[3].y = f3;
-    if (mx && !lo) g[6].x = f6;
-    if (my && !lo) g[6].y = f6;
-    if (mx && !hi) g[7].x = f7;
-    if (my && !hi) g[7].y = f7;
-  }
-
-  // ---- walls ----
-  // a stage field on solid row q: the wall temperature; the top ghost of an adiabatic
-  // column copies row ny - 1 (`below`, the row swept before)
-  __device__ __forceinline__ V wall_T(int q, V below) const {
-    float w[2];
-#pragma unroll
-    for (int j = 0; j < 2; j++) {
-      const int x = XO ? c0 + j : (j ? x0 + o1 : x0);
-      w[j] = q < 0 ? wall_T_dev(p, x) : wall_T_top_dev(p, x);
-      if (!XO && q >= 0 && p.adiabatic && wall_adiabatic(p, x, true)) w[j] = j ? below.y : below.x;
-    }
-    return vset(w[0], w[1]);
-  }
-  // the bottom ghost of an adiabatic column copies row 0: once row 0 has its value v, it goes
-  // into the ghost row's slot
-  __device__ __forceinline__ void mirror_bottom(V &slot, V v) const {
-    if (!XO && p.adiabatic) {
-      if (wall_adiabatic(p, x0, false)) slot.x = v.x;
-      if (wall_adiabatic(p, x0 + o1, false)) slot.y = v.y;
-    }
-  }
   // the ghosts of row q of a new stage field v; below: the field's row q - 1
   __device__ __forceinline__ V stage_ghosts(bool near, int q, V v, V &below) const {
     if (near) {
-      if ((unsigned)q >= (unsigned)p.ny) v = wall_T(q, below);
-      if (!XO && q == 0) mirror_bottom(below, v);
+      if ((unsigned)q >= (unsigned)p.ny) v = this->wall_T(q, below);
+      if (!XO && q == 0) this->mirror_bottom(below, v);
     }
     return v;
   }
 
-  // ---- loads ----
-  // element at byte offset b (32-bit) from a uniform base
-  template <class X>
-  static __device__ __forceinline__ X *at(X *base, unsigned b) {
-    return const_cast<X *>(
-        reinterpret_cast<const X *>(reinterpret_cast<const char *>(base) + b));
-  }
-  // issue the loads of row r; near: it may be a wall row or next to one
-  __device__ __forceinline__ void load_row(bool near, int r) {
-    if (YW && near && (unsigned)r >= (unsigned)p.ny) return;
-    const int ry = YW ? r : modi(r, p.ny);
-    const unsigned R = (unsigned)(ry * p.pitch + x0);  // element offset in a plane
-    if (YW && near && (ry == 0 || ry == p.ny - 1)) {
-      // next to a wall: links from the solid row come from the node's own opposite
-      // population (half-way bounce-back; the weights of the two are the same)
-#pragma unroll
-      for (int i = 0; i < 9; i++) {
-        const bool back = (ey(i) == 1 && ry == 0) || (ey(i) == -1 && ry == p.ny - 1);
-        const int e = back ? 0 : ex(i);
-        const T *b = gs + (back ? opp(i) * p.plane : i * p.plane - ey(i) * p.pitch) + R;
-        const int a = e == 0 ? 0 : (e == 1 ? oW : o1);
-        const int c = e == 0 ? o1 : (e == 1 ? 0 : oE);
-        g[i] = vset(pop<ST>(b + a, i), pop<ST>(b + c, i));
-      }
-    } else {
-      // rows below and above: offsets of their own where the rows wrap
-      const unsigned Rm = YW ? R - p.pitch : (unsigned)(modi(ry - 1, p.ny) * p.pitch + x0);
-      const unsigned Rp = YW ? R + p.pitch : (unsigned)(modi(ry + 1, p.ny) * p.pitch + x0);
-#pragma unroll
-      for (int i = 0; i < 9; i++) {
-        const T *b = gs + i * p.plane;
-        const unsigned o = (ey(i) == 0 ? R : (ey(i) == 1 ? Rm : Rp)) * E;
-        if (XO) {
-          // (planes 1 .. 8: a neighbour element is in bounds at the ends of the array too)
-          if (ex(i) == 0) {
-            g[i] = pop2<ST>(at(b, o), i);
-          } else {
-            g[i] = vset(pop<ST>(at(b, o) - ex(i), i), pop<ST>(at(b, o) - ex(i) + 1, i));
-          }
-        } else if (ex(i) == 0) {
-          g[i] = vec ? pop2<ST>(at(b, o), i)
-                     : vset(pop<ST>(at(b, o), i), pop<ST>(at(b, o) + o1, i));
-        } else {
-          g[i] = vset(pop<ST>(at(b, o) + (ex(i) == 1 ? oW : o1), i),
-                      pop<ST>(at(b, o) + (ex(i) == 1 ? 0 : oE), i));
-        }
-      }
-    }
-    const float *t = at(Tin, 4u * R);
-    Tn = vec ? *reinterpret_cast<const float2 *>(t) : vset(t[0], t[o1]);
-  }
-
-  // ---- energy equation ----
   __device__ __forceinline__ void put_own(int j, const Own &o) {
     float4 *d = own_s + (j & 3) * 96;
     d[0] = make_float4(o.nux.x, o.nux.y, o.nuy.x, o.nuy.y);
@@ -434,15 +82,6 @@ struct Sweep {
     return Own{vset(a.x, a.y), vset(a.z, a.w), vset(b.x, b.y),
                vset(b.z, b.w), vset(c.x, c.y), vset(c.z, c.w)};
   }
-  // K(T) of Eq. 16 (see rk_rate): -us.g + cl L - E1 x - E2 s
-  __device__ __forceinline__ V rate(V dn, V c, V up, const Own &o) const {
-    const Sten t = stencil(dn, c, up, false);
-    const V lap = t.es + vfma(kl(-5.0f), c, t.a);
-    const V x = vfma(kp(k.inv_Tc), c, kp(k.xr));  // T/Tc > 0 on fluid nodes
-    const V s = x * vrsqrt(x);
-    return vfma(o.nE2, s, vfma(o.nE1, x, vfma(o.cl, lap, vfma(o.nux, t.gx, o.nuy * t.gy))));
-  }
-
   // One row step: row r = Y0 - HR + j, P = j & 1.  Every value is computed in the straight
   // line, and a rare case (wall rows, open ends) overwrites it afterwards, so that no value
   // that is carried on has two sources to be copied together.
@@ -455,82 +94,31 @@ struct Sweep {
     const bool near = YW && (unsigned)(r - NW) >= span;
     // ---------------- S0: row r ----------------
     const bool solid = near && (unsigned)r >= uny;
-    if (XO && ends && !solid) {
-      if (e_in) inlet_fix(r);
-      if (e_out) outlet_fix(r);
-      if (e_in) Tn = inlet_set(Tn, p.T_inlet_dev);
-    }
+    if (XO && ends && !solid) this->open_ends(r);
     V T_r = Tn;
-    V *n = m[P];
-    {
-      // the moments n = M g (Eq. 6) from sums and differences of opposite directions
-      const V s13 = g[1] + g[3], s24 = g[2] + g[4], s57 = g[5] + g[7], s68 = g[6] + g[8];
-      const V d13 = g[1] - g[3], d24 = g[2] - g[4], d57 = g[5] - g[7], d68 = g[6] - g[8];
-      const V sa = s13 + s24, sd = s57 + s68, f0 = g[0];
-      const V dx = d57 - d68, dy = d57 + d68;
-      n[0] = (f0 + sa) + sd;
-      n[1] = vfma(kl(-2.0f), sd, vfma(kl(4.0f), f0, sa));  // -n1
-      n[2] = vfma(kl(-2.0f), sa, vfma(kl(4.0f), f0, sd));
-      n[3] = d13 + dx;
-      n[4] = vfma(kl(-2.0f), d13, dx);
-      n[5] = d24 + dy;
-      n[6] = vfma(kl(-2.0f), d24, dy);
-      n[7] = s13 - s24;
-      n[8] = s57 - s68;
-    }
-    const V drho = n[0];
+    this->moments(m[P]);
+    const V drho = m[P][0];
     V psi_r = vdup(0.0f), cfx_r, cfz_r;
-    bool neg0 = false, neg1 = false, neg = false;
-    if (MP || TH) {
-      // Peng-Robinson differences (see pseudopotential_dev) and the energy coefficients of
-      // the density: E1 / (3 div u), E2 / (3 div u)
-      const V rho = kp(k.rho_ref) + drho;
-      const V br = k1(k.b) * rho;
-      const V inv1 = vrcp(kl(1.0f) - br);
-      const V invD = vrcp(vfma(br, kl(2.0f) - br, kl(1.0f)));
-      if (TH) {
-        cfz_r = (k1(k.akap1_cv3) * rho) * invD;
-        cfx_r = vfma(k1(k.nkappa_r), cfz_r, k1(k.RTc_cv3) * inv1);
-      }
-      if (MP) {
-        const V s = vsqrt(vfma(kp(k.inv_Tc), T_r, kp(k.xr)));
-        const V ds = (kp(k.inv_Tc) * T_r) * vrcp(k1(k.sr) + s);
-        const V rr = vfma(k1(k.nkappa), s, k1(k.kappa1r));  // r(T) + r(T_ref)
-        const V gg = vfma(k1(k.ps_g), rho, kp(k.rho_ref));
-        const V tR = inv1 * vfma(k1(k.ps_RT) * T_r, rho, k1(k.ps_R) * drho);
-        const V tA = invD * vfma((k1(k.ps_phi) * ds) * rr, rho * rho, (k1(k.ps_B) * drho) * gg);
-        const V dpsi2 = vfma(k1(k.ps_3), drho, tR - tA);
-        const V psi2 = k1(k.psi_r2) + dpsi2;
-        const V root = vsqrt(vset(fmaxf(psi2.x, 0.0f), fmaxf(psi2.y, 0.0f)));
-        psi_r = dpsi2 * vrcp(k1(k.psi_den) + root);
-        // a negative argument gives psi = 0 and a status bit (a ghost's populations include
-        // unfixed placeholders, a solid row's are left over)
-        neg0 = !(psi2.x >= 0.0f);
-        neg1 = !(psi2.y >= 0.0f);
-        psi_r.x = neg0 ? -p.psi_r : psi_r.x;
-        psi_r.y = neg1 ? -p.psi_r : psi_r.y;
-        neg = neg0 || neg1;
-      }
-    }
+    bool neg0 = false, neg1 = false;
+    this->state(drho, T_r, psi_r, cfx_r, cfz_r, neg0, neg1);
+    // (a ghost's populations include unfixed placeholders, a solid row's are left over)
+    bool neg = neg0 || neg1;
     V dr = drho, dt = T_r;
     if (XO && ends) {
-      if (ghost(0)) dr.x = dt.x = 0.0f;
-      if (ghost(1)) dr.y = dt.y = 0.0f;
-      if (MP) neg = (neg0 && !ghost(0)) || (neg1 && !ghost(1));
+      if (this->ghost(0)) dr.x = dt.x = 0.0f;
+      if (this->ghost(1)) dr.y = dt.y = 0.0f;
+      if (MP) neg = (neg0 && !this->ghost(0)) || (neg1 && !this->ghost(1));
     }
     if (near) {
       if (solid) {
         psi_r = dr = dt = vdup(0.0f);
-        T_r = wall_T(r, T1);
+        T_r = this->wall_T(r, T1);
         neg = false;
       }
-      if (TH && !XO && r == 0) mirror_bottom(T1, T_r);
+      if (TH && !XO && r == 0) this->mirror_bottom(T1, T_r);
     }
-    if (MP) st |= neg ? ST_PSI_NEG : 0u;
-    drho_min = fminf(drho_min, fminf(dr.x, dr.y));
-    drho_max = fmaxf(drho_max, fmaxf(dr.x, dr.y));
-    dT_min = fminf(dT_min, fminf(dt.x, dt.y));
-    if (j + 1 < J) load_row(near, r + 1);
+    this->track(dr, dt, neg);
+    if (j + 1 < J) this->load_row(near, r + 1);
     // (keeps the loads here: moved down to the end of the step they are not back in time;
     // 4096 x 512: 53.7 against 64.6 us per update)
     __syncwarp();
@@ -539,111 +127,23 @@ struct Sweep {
     V u_x = vdup(0.0f), u_y = vdup(0.0f), cl_q = vdup(0.0f);
     if (!WARM || j >= 2) {
       const int q = r - 1;
-      const V *n = m[Q];
-      const V drho = n[0];
-      V Fx = vdup(0.0f), Fy = vdup(0.0f), fm2 = vdup(0.0f);
-      if (MP) {
-        const Sten t = stencil(psi[P], psi[Q], psi_r, true);
-        const V gpsi = vfma(k1(k.G3), psi[Q], k1(k.G3r));  // -G psi / 3
-        Fx = gpsi * t.gx;
-        Fy = gpsi * t.gy;
-        V qy = t.gy;
-        if (near && (q == 0 || q == p.ny - 1)) {
-          // wall neighbours (psi of a solid row is 0 in the stencil): Eq. 14, see
-          // interaction_force; Sy = 3 sum_solid w e_y
-          const float Sy = (q == p.ny - 1 ? 1.5f : 0.0f) - (q == 0 ? 1.5f : 0.0f);
-          float wc[2];
-#pragma unroll
-          for (int i = 0; i < 2; i++) {
-            const float Tq = i ? T1.y : T1.x, pc = i ? psi[Q].y : psi[Q].x;
-            unsigned unused = 0u;
-            wc[i] = p.rho_w > 0.0f
-                        ? p.G * p.psi_r - p.Gw * pseudopotential(p, p.rho_w, p.T_ref + Tq, unused)
-                        : p.wall_r - p.Gw * pc;
-          }
-          const V ws = kl(1.0f / 3.0f) * (vdup(p.psi_r) + psi[Q]) * vset(wc[0], wc[1]);
-          Fy = vfma(ws, vdup(Sy), Fy);
-          qy = vfma(vdup(-p.psi_r), vdup(Sy), qy);
-        }
-        fm2 = vfma(t.gx, t.gx, qy * qy);
-      }
-      if (has_g) {
-        const V rv = vdup(p.drho_ref_g) + drho;  // rho - rho_v of Eq. 15
-        Fx = Fx + rv * vdup(p.gx) * vdup(sc.gcos);
-        Fy = Fy + rv * vdup(p.gy) * vdup(sc.gcos);
-      }
-      const V rho = kp(k.rho_ref) + drho;
+      const V (&n)[9] = m[Q];
+      V Fx, Fy, fm2;
+      this->forces(q, near && (q == 0 || q == p.ny - 1), psi[P], psi[Q], psi_r, T1, n[0], Fx, Fy,
+                   fm2);
+      const V rho = kp(k.rho_ref) + n[0];
       const V ir = vrcp(rho);
       const V jx = vfma(kl(0.5f), Fx, n[3]), jy = vfma(kl(0.5f), Fy, n[5]);  // rho u
       u_x = jx * ir;
       u_y = jy * ir;
       if (TH) cl_q = k1(k.lam23_cv) * ir;
-      if ((unsigned)(q - Y0) < (unsigned)(ye - Y0)) {
-        // moment-space collision (see collide): a_k = (m*_k - rho_ref c_k) / D_k
-        const V uxF = u_x * Fx, uyF = u_y * Fy, uxj = jx * u_x, uyj = jy * u_y;
-        const V uF = uxF + uyF, uu = uxj + uyj;
-        const V dF = uxF - uyF, dj = uxj - uyj, xF = vfma(u_x, Fy, u_y * Fx), xj = jx * u_y;
-        V a7, a8;
-        if (tau_const) {
-          a7 = vfma(k1(k.kn2), dF, vfma(kp(k.kn1), dj, kp(k.kn0) * n[7]));
-          a8 = vfma(k1(k.kn3), xF, vfma(kp(k.kn1), xj, kp(k.kn0) * n[8]));
-        } else {
-          const float fx = fminf(fmaxf((rho.x - p.rho_g) * p.inv_drho, 0.0f), 1.0f);
-          const float fy = fminf(fmaxf((rho.y - p.rho_g) * p.inv_drho, 0.0f), 1.0f);
-          // c = 0.25 s_nu of Eq. 5
-          const V c = kl(0.25f) * vrcp(vset(p.tau_g + fx * p.dtau, p.tau_g + fy * p.dtau));
-          const V ca = kl(0.25f) - c;
-          a7 = vfma(kl(0.5f) - c, dF, vfma(c, dj, ca * n[7]));
-          a8 = vfma(vfma(kl(-0.5f), c, kl(0.25f)), xF, vfma(c, xj, ca * n[8]));
-        }
-        const V a0 = k1(1.0f / 9.0f) * drho;
-        const V a1 = vfma(k1(k.k14), fm2, vfma(k1(k.k13), uF, vfma(k1(k.k12), uu,
-                              vfma(k1(k.k11), drho, k1(k.nk10) * n[1]))));
-        const V a2 = vfma(k1(k.k24), fm2, vfma(k1(k.k23), uF, vfma(k1(k.k22), uu,
-                              vfma(k1(k.k21), drho, k1(k.k20) * n[2]))));
-        const V a3 = k1(1.0f / 6.0f) * (n[3] + Fx), a5 = k1(1.0f / 6.0f) * (n[5] + Fy);
-        const V a4 = vfma(kp(k.kq2), Fx, vfma(kp(k.kq1), jx, kp(k.kq0) * n[4]));
-        const V a6 = vfma(kp(k.kq2), Fy, vfma(kp(k.kq1), jy, kp(k.kq0) * n[6]));
-        const KL m2 = kl(-2.0f);
-        const V b_ax = vfma(m2, a2, a0 - a1), b_dg = vfma(kl(2.0f), a1, a0) + a2;
-        const V px = vfma(m2, a4, a3), py = vfma(m2, a6, a5);
-        const V tx = a3 + a4, ty = a5 + a6;
-        const V qs = tx + ty, qd = ty - tx;
-        const V axp = b_ax + a7, axm = b_ax - a7, dgp = b_dg + a8, dgm = b_dg - a8;
-        V o[9];
-        o[0] = vfma(kl(4.0f), a2 - a1, a0);
-        o[1] = axp + px;
-        o[2] = axm + py;
-        o[3] = axp - px;
-        o[4] = axm - py;
-        o[5] = dgp + qs;
-        o[6] = dgm + qd;
-        o[7] = dgp - qs;
-        o[8] = dgm - qd;
-        V ck = u_x * u_y;  // not finite when either is not
-        if (XO ? e_out : oddx) {
-          // odd nx: the padding column stays zero
-          if (oddx) {
-            ck.y = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 9; i++) o[i].y = 0.0f;
-          }
-        }
-        // whole pairs: with the energy equation the pairs at the ends of the output columns
-        // hold one halo column each, whose populations are complete here too; the
-        // neighbouring warp stores the same bits
-        if (outp) {
-          chk = chk + ck;
-          const unsigned so = (unsigned)((YW ? q : modi(q, p.ny)) * p.pitch + c0) * E;
-#pragma unroll
-          for (int i = 0; i < 9; i++) ST::store2(at(gout + i * p.plane, so), o[i].x, o[i].y, i);
-        }
-      }
+      if ((unsigned)(q - Y0) < (unsigned)(ye - Y0))
+        this->collide_store(q, n, rho, jx, jy, u_x, u_y, Fx, Fy, fm2);
       if (TH) {
         // the velocity inlet's ghost holds the inlet velocity
         if (XO && e_in) {
-          u_x = inlet_set(u_x, sc.u_in);
-          u_y = inlet_set(u_y, 0.0f);
+          u_x = this->inlet_set(u_x, sc.u_in);
+          u_y = this->inlet_set(u_y, 0.0f);
         }
         if (near && (unsigned)q >= uny) u_x = u_y = vdup(0.0f);
       }
@@ -651,46 +151,26 @@ struct Sweep {
     if (TH) {
       if (!WARM || j >= 4) {
         // ---------------- S2: row r-2 (div u, h1) ----------------
-        const KL q4 = kl(0.25f);
-        const K1 n3 = k1(-1.0f / 3.0f);
-        V sx = vfma(q4, u_x + ux[Q], ux[P]), dy = u_y - uy[Q];
-        float w, e, dw, de;
-        neighbours2(sx, dy, p.p_inlet != 0, w, e, dw, de);
-        const V nd = kl(-1.0f) * (vset(sx.y - w, e - sx.x) + vfma(q4, vset(dy.y + dw, de + dy.x), dy));
-        Own o{n3 * ux[P], n3 * uy[P], cl, T2, cfx[P] * nd, cfz[P] * nd};
-        // the inlet ghost keeps T_inlet through the stages: no rate there
-        if (XO && ends && c0 == -2) o.nux.y = o.nuy.y = o.cl.y = o.nE1.y = o.nE2.y = 0.0f;
+        const Own o = this->own_values(ux[Q], ux[P], u_x, uy[Q], uy[P], u_y, cl, T2, cfx[P], cfz[P]);
         put_own(j, o);
-        const V h1 = rate(T3, T2, T1, o);
+        const V h1 = this->rate(T3, T2, T1, o);
         const V v2 = stage_ghosts(near, r - 2, vfma(kl(0.5f), h1, T2), K2[Q]);
         if (!WARM || j >= 6) {
           // ---------------- S3: row r-3 (h2) ----------------
           const Own o3 = get_own(j - 1);
-          const V h2 = rate(K2[P], K2[Q], v2, o3);
+          const V h2 = this->rate(K2[P], K2[Q], v2, o3);
           const V v3 = stage_ghosts(near, r - 3, vfma(kl(0.5f), h2, o3.Tb), K3[P]);
           if (!WARM || j >= 8) {
             // ---------------- S4: row r-4 (h3) ----------------
             const Own o4 = get_own(j - 2);
-            const V h3 = rate(K3[Q], K3[P], v3, o4);
+            const V h3 = this->rate(K3[Q], K3[P], v3, o4);
             const V v4 = stage_ghosts(near, r - 4, o4.Tb + h3, K4[Q]);
             if (!WARM) {
               // ---------------- S5: row r-5 (h4, new temperature) ----------------
               const Own o5 = get_own(j - 3);
-              const V h4 = rate(K4[P], K4[Q], v4, o5);
+              const V h4 = this->rate(K4[P], K4[Q], v4, o5);
               const V Tnew = vfma(k1(1.0f / 6.0f), acc3 + h4, o5.Tb);
-              const unsigned so = 4u * (unsigned)((YW ? r - 5 : modi(r - 5, p.ny)) * p.pitch + c0);
-              float *d = at(Tout, so);
-              if (out0 && out1) {
-                chk = chk + Tnew;
-                dT_min = fminf(dT_min, fminf(Tnew.x, Tnew.y));
-                *reinterpret_cast<float2 *>(d) = Tnew;
-              } else if (out0 || out1) {
-                const float v = out0 ? Tnew.x : Tnew.y;
-                chk.x += v;
-                dT_min = fminf(dT_min, v);
-                if (out0) d[0] = v;
-                if (out1) at(Tout, so + 4u)[0] = v;
-              }
+              this->store_T(r - 5, Tnew);
             }
             acc3 = vfma(kl(2.0f), h3, acc2);
             K4[P] = vcopy(v4);
@@ -716,7 +196,7 @@ struct Sweep {
   __device__ __forceinline__ void run(unsigned *status) {
     const int J = ye - Y0 + 2 * HR;
     constexpr int JW = 2 * HR;  // steps until every stage has a row (even, below J)
-    load_row(true, Y0 - HR);
+    this->load_row(true, Y0 - HR);
 #pragma unroll 1
     for (int j = 0; j < JW; j += 2) {
       step<0, true>(j, J);
@@ -729,11 +209,7 @@ struct Sweep {
       step<1, false>(j, J);
       if (++j >= J) break;
     }
-    if (!isfinite(chk.x + chk.y)) st |= ST_NAN;
-    if (!(p.rho_ref + drho_min > 0.0f)) st |= ST_RHO_NONPOS;
-    if (!(p.eos_b * (p.rho_ref + drho_max) < 1.0f)) st |= ST_EOS_POLE;
-    if (!(p.T_ref + dT_min > 0.0f)) st |= ST_T_NONPOS;
-    set_status(status, st);
+    this->finish(status);
   }
 };
 

@@ -9,8 +9,8 @@ cudaError_t sweep_f16_occupancy(const DevParams &p, int *occ) {
 
 cudaError_t sweep_f16_launch(const DevParams &p, const void *gs, void *gout, const float *Tin,
                              float *Tout, unsigned *status, const StepScalars *sc,
-                             const SweepTiling &tl, cudaStream_t s) {
-  return sweep_launch_t<StoreF16>(p, gs, gout, Tin, Tout, status, sc, tl, s);
+                             const StepScalars &val, const SweepTiling &tl, cudaStream_t s) {
+  return sweep_launch_t<StoreF16>(p, gs, gout, Tin, Tout, status, sc, val, tl, s);
 }
 
 }  // namespace lbm

@@ -19,57 +19,13 @@ constexpr int SNT = 32 * SW;
 // against 575 us, 16-bit storage 987 against 720 us); 16 warps (128 registers) spill.
 constexpr int SMIN = 3;
 
-SweepConsts sweep_consts(const DevParams &p) {
-  SweepConsts k;
-  k.rho_ref = p.rho_ref;
-  k.b = p.eos_b;
-  k.inv_Tc = p.inv_Tc;
-  k.xr = p.xr;
-  k.sr = p.sr;
-  k.nkappa = -p.kappa;
-  k.kappa1r = p.kappa1 + p.rphi_r;
-  k.ps_g = p.ps_g;
-  k.ps_RT = p.ps_RT;
-  k.ps_R = p.ps_R;
-  k.ps_phi = p.ps_phi;
-  k.ps_B = p.ps_B;
-  k.ps_3 = p.ps_3;
-  k.psi_r2 = p.psi_r2;
-  // the denominator psi + psi_r stays positive where both vanish (the quotient is 0 there)
-  k.psi_den = std::max(p.psi_r, 1e-30f);
-  k.akap1_cv3 = p.akap1_cv3;
-  k.nkappa_r = -p.kappa_r;
-  k.RTc_cv3 = p.RTc_cv3;
-  k.lam23_cv = p.lam23_cv;
-  k.G3 = p.G3;
-  k.G3r = p.G3r;
-  k.nk10 = -p.k1[0];
-  k.k11 = p.k1[1];
-  k.k12 = p.k1[2];
-  k.k13 = p.k1[3];
-  k.k14 = p.k1[4];
-  k.k20 = p.k2[0];
-  k.k21 = p.k2[1];
-  k.k22 = p.k2[2];
-  k.k23 = p.k2[3];
-  k.k24 = p.k2[4];
-  k.kq0 = p.kq[0];
-  k.kq1 = p.kq[1];
-  k.kq2 = p.kq[2];
-  k.kn0 = p.kn[0];
-  k.kn1 = p.kn[1];
-  k.kn2 = p.kn[2];
-  k.kn3 = p.kn[3];
-  return k;
-}
-
 template <bool YW, bool XO, bool TH, bool MP, class ST>
 __global__ void __launch_bounds__(SNT, SMIN)
     k_sweep(const __grid_constant__ DevParams p, const __grid_constant__ SweepConsts k,
             const typename ST::T *gs, typename ST::T *gout, const float *Tin, float *Tout,
-            unsigned *status, const StepScalars *__restrict__ sc) {
+            unsigned *status, const StepScalars *__restrict__ sc, const StepScalars val) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const StepScalars ssc = *sc;
+  const StepScalars ssc = sc ? *sc : val;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const int Y0 = (int)(((long long)blockIdx.y * p.ny) / gridDim.y);
   const int ye = (int)(((long long)(blockIdx.y + 1) * p.ny) / gridDim.y);
@@ -84,7 +40,7 @@ __global__ void __launch_bounds__(SNT, SMIN)
 
 template <class ST>
 using SweepFn = void (*)(DevParams, SweepConsts, const typename ST::T *, typename ST::T *,
-                         const float *, float *, unsigned *, const StepScalars *);
+                         const float *, float *, unsigned *, const StepScalars *, StepScalars);
 
 template <class ST>
 SweepFn<ST> sweep_variant(const DevParams &p) {
@@ -107,7 +63,7 @@ int sweep_cols(int strips) { return (strips + SW - 1) / SW; }
 template <class ST>
 cudaError_t sweep_launch_t(const DevParams &p, const void *gs, void *gout, const float *Tin,
                            float *Tout, unsigned *status, const StepScalars *sc,
-                           const SweepTiling &tl, cudaStream_t s) {
+                           const StepScalars &val, const SweepTiling &tl, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)sweep_cols(tl.strips), (unsigned)tl.chunks);
   cfg.blockDim = dim3(SNT);
@@ -119,7 +75,7 @@ cudaError_t sweep_launch_t(const DevParams &p, const void *gs, void *gout, const
   cfg.numAttrs = tl.pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, sweep_variant<ST>(p), p, sweep_consts(p),
                             static_cast<const typename ST::T *>(gs),
-                            static_cast<typename ST::T *>(gout), Tin, Tout, status, sc);
+                            static_cast<typename ST::T *>(gout), Tin, Tout, status, sc, val);
 }
 
 template <class ST>

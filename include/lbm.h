@@ -234,9 +234,13 @@ int lbm_droplet_stats(const double *rho, int nx, int ny, double threshold, doubl
    A batch groups lattices that share the boundary modes (x_bc class, y_bc), the
    thermal and multiphase switches and the storage, and that use the fused kernel or
    the two-pass path (LBM_KERNEL_AUTO gives one of the two);
-   sizes and all other parameters may differ.  Each step is one launch whose
-   resident CTAs take tiles of all lattices from one work-list (largest lattices
-   first) through an atomic counter.  The batch borrows the lattices: they stay
+   sizes and all other parameters may differ.  Each step is one launch over the tiles of
+   all lattices, largest lattices first: with the energy equation and the pseudopotential
+   by independent warps (one launch for every 48 lattices), each on a strip of 54 columns of
+   a row chunk; in the other modes, with a tiling of their own (lbm_batch_set_tiling) and
+   with 16-bit storage, unless every lattice is on the library's kernel choice, by resident
+   CTAs that take tiles from one work-list through an atomic counter.  The
+   batch borrows the lattices: they stay
    owned by the caller, must outlive the batch, and while batched should be advanced
    only through lbm_batch_step (their own t, buffers and status words advance).
    A lattice's fields after lbm_batch_step equal those after lbm_step alone. */
@@ -253,13 +257,13 @@ int lbm_batch_set_graph(lbm_batch_h b, int enable);
 /* Output rows per tile (the work-list granularity).  The default, chosen at creation, is the
    height among 128, 96, 64, 48, 32, 24 and 16 rows whose work-list a greedy schedule over
    the resident CTAs finishes first; if that leaves fewer tiles than SMs, heights down to
-   1 row compete, with row steps slower the more tiles share an SM.  A launch has one CTA
-   per tile when there are fewer tiles than resident CTAs. */
+   1 row compete, with row steps slower the more tiles share an SM. */
 int lbm_batch_set_tile_rows(lbm_batch_h b, int rows);
 /* Set the tiling: output rows and columns per tile and lattice columns per thread (1, or 2
    when the batch's modes include the energy equation and the pseudopotential forces; cols
-   at most 118 with one column per thread, an even number up to 244 with two).
-   LBM_ERR_ARG otherwise.  Results do not depend on the tiling. */
+   at most 118 with one column per thread, an even number up to 244 with two) of the
+   work-list kernel, which runs the batch from then on.  LBM_ERR_ARG otherwise.  Results do
+   not depend on the tiling. */
 int lbm_batch_set_tiling(lbm_batch_h b, int rows, int cols, int cols_per_thread);
 int lbm_batch_tiling(lbm_batch_h b, int *rows, int *cols, int *cols_per_thread);
 /* The library's autotuner: times tilings with steps_per_candidate timed updates each (plus

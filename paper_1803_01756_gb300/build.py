@@ -30,7 +30,7 @@ _FAST = ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]
 PER_FILE = {"lbm_fused.cu": _FAST + ["-Xptxas=--register-usage-level=8"]}
 PER_FILE.update({f + ".cu": _FAST for f in (
     "lbm_fused_c2", "lbm_fused_batch", "lbm_twopass", "lbm_sweep", "lbm_sweep_f16",
-    "lbm_sweep_bf16", "lbm_tile", "lbm_tile_f16", "lbm_tile_bf16")})
+    "lbm_sweep_bf16", "lbm_sweep_batch", "lbm_sweep_batch_f16", "lbm_sweep_batch_bf16", "lbm_tile", "lbm_tile_f16", "lbm_tile_bf16")})
 _lock = threading.Lock()
 
 

@@ -19,6 +19,11 @@ struct lbm_batch {
   int tile_cols = 0;               // output columns per tile (even with two columns per thread)
   int cpt = 1;                     // lattice columns per thread of the batched kernel
   int grid_of[3] = {0, 0, 0};      // resident CTAs with 1 and 2 columns per thread (0: none)
+  // The warp sweep runs the batch until a tiling of the CTA kernel is asked for
+  // (lbm_batch_set_tiling, lbm_batch_autotune): its tiles are a warp's strip of a row chunk.
+  int sweep_slots = 0;             // its resident CTAs (0: the modes have no such kernel)
+  bool sweep = false;
+  std::vector<lbm::SweepBatchItem> items;
   int ntiles = 0, grid = 0, sms = 1;
   BatchChannel *d_ch[2] = {nullptr, nullptr};  // tables for even and odd steps of a call
   std::vector<BatchChannel> h_ch[2];
@@ -39,8 +44,9 @@ namespace {
 
 using lbm_host::cuda_fail;
 
-int tiles_of(const lbm_lattice *h, int rows, int cols) {
+int tiles_of(const lbm_batch *b, const lbm_lattice *h, int rows, int cols) {
   const int H = std::min(rows, h->ny);
+  if (b->sweep) return lbm::sweep_batch_strips(h->nx) * ((h->ny + H - 1) / H);
   return ((h->nx + cols - 1) / cols) * ((h->ny + H - 1) / H);
 }
 
@@ -54,29 +60,36 @@ void drop_graph(lbm_batch *b) {
 // Work-list layout for the current tile height: lattices with the most work first
 void layout(lbm_batch *b) {
   std::stable_sort(b->lat.begin(), b->lat.end(), [&](const lbm_lattice *x, const lbm_lattice *y) {
-    return (long long)tiles_of(x, b->tile_rows, b->tile_cols) * x->nx >
-           (long long)tiles_of(y, b->tile_rows, b->tile_cols) * y->nx;
+    return (long long)tiles_of(b, x, b->tile_rows, b->tile_cols) * x->nx >
+           (long long)tiles_of(b, y, b->tile_rows, b->tile_cols) * y->nx;
   });
   b->ntiles = 0;
-  for (auto *h : b->lat) b->ntiles += tiles_of(h, b->tile_rows, b->tile_cols);
-  b->grid = b->grid_of[b->cpt];
+  for (auto *h : b->lat) b->ntiles += tiles_of(b, h, b->tile_rows, b->tile_cols);
+  b->grid = b->sweep ? b->sweep_slots * lbm::sweep_batch_warps() : b->grid_of[b->cpt];
+  b->items.clear();
+  if (b->sweep)
+    for (auto *h : b->lat)
+      b->items.push_back({&h->dp, (h->ny + b->tile_rows - 1) / b->tile_rows});
   drop_graph(b);
 }
 
-// Greedy list schedule of the work-list at tile height H over `grid` CTA slots (tiles in
-// launch order, each taken by the first free slot, a tile costing its row steps H + 15):
-// returns the makespan in row steps and the number of tiles.
+// Greedy list schedule of the work-list at tile height H over the resident CTAs (CTAs in
+// launch order, each taken by the first free slot, costing its row steps: H + 15, in the warp
+// sweep H + 10): returns the makespan in row steps and the number of tiles.
 double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, int H,
                 long long &ntiles) {
   const int W = b->tile_cols;
   std::priority_queue<double, std::vector<double>, std::greater<double>> slots;
-  for (int k = 0; k < b->grid; k++) slots.push(0.0);
+  const int resident = b->sweep ? b->sweep_slots : b->grid;
+  const double fill = b->sweep ? 10.0 : 15.0;
+  for (int k = 0; k < resident; k++) slots.push(0.0);
   double makespan = 0.0;
   ntiles = 0;
   for (const lbm_lattice *h : order) {
-    const int rows = std::min(H, h->ny), strips = (h->nx + W - 1) / W;
+    const int rows = std::min(H, h->ny);
+    const int strips = b->sweep ? lbm::sweep_batch_cols(h->nx) : (h->nx + W - 1) / W;
     for (int y0 = 0; y0 < h->ny; y0 += rows) {
-      const double len = std::min(rows, h->ny - y0) + 15.0;
+      const double len = std::min(rows, h->ny - y0) + fill;
       for (int x = 0; x < strips; x++) {
         const double t = slots.top() + len;
         slots.pop();
@@ -85,6 +98,7 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
         ntiles++;
       }
     }
+    if (b->sweep) ntiles += (long long)(lbm::sweep_batch_strips(h->nx) - strips) * ((h->ny + rows - 1) / rows);
   }
   return makespan;
 }
@@ -100,7 +114,8 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
 // with 16-bit storage, four: one CTA alone is bound by the latency of its row step, a
 // full SM shares the issue slots), so that a few small lattices spread over the SMs
 // (200 x 50 alone: 1 row, 17.0 against 39.3 us per update with 16; 1024 x 128: 4 rows,
-// 22.8 against 39.6 us).
+// 22.8 against 39.6 us).  The figures are the CTA kernel's; the warp sweep is scheduled by
+// the same rule with its own row steps and CTAs.
 int default_rows(const lbm_batch *b) {
   static const int tall[] = {128, 96, 64, 48, 32, 24, 16};
   static const int small[] = {16, 12, 8, 6, 4, 3, 2, 1};
@@ -123,7 +138,7 @@ int default_rows(const lbm_batch *b) {
     }
   }
   if (best_tiles >= b->sms) return best;
-  const int occ = std::max(1, std::min(4, b->grid / b->sms));
+  const int occ = std::max(1, std::min(4, (b->sweep ? b->sweep_slots : b->grid) / b->sms));
   const double *kStep = occ >= 4 ? kStep4 : kStep3;
   best_cost = 0.0;
   for (int H : small) {
@@ -163,7 +178,7 @@ int upload_tables(lbm_batch *b, cudaStream_t s) {
       c.strips = (h->nx + W - 1) / W;
       c.tile_begin = begin;
     }
-    begin += tiles_of(h, b->tile_rows, b->tile_cols);
+    begin += tiles_of(b, h, b->tile_rows, b->tile_cols);
   }
   const size_t bytes = sizeof(BatchChannel) * b->lat.size();
   for (int par = 0; par < 2; par++)
@@ -174,18 +189,21 @@ int upload_tables(lbm_batch *b, cudaStream_t s) {
 // CTAs of one launch: the resident grid, or one per tile when there are fewer tiles
 int launch_grid(const lbm_batch *b) { return std::min(b->grid, b->ntiles); }
 
-int launch_one(lbm_batch *b, int k, cudaStream_t s) {
+// step k of a chunk with the buffers of table par
+int launch_one(lbm_batch *b, int k, int par, cudaStream_t s) {
   const int n = (int)b->lat.size();
-  return cuda_fail(lbm::launch_fused_batch(b->mode, b->storage, b->cpt, b->d_ch[k & 1], n,
-                                           b->d_sc + (size_t)k * n, b->ntiles, b->d_counter,
-                                           launch_grid(b), s));
+  const StepScalars *sc = b->d_sc + (size_t)k * n;
+  if (b->sweep)
+    return cuda_fail(lbm::launch_sweep_batch(b->storage, b->items.data(), n, b->d_ch[par], sc, s));
+  return cuda_fail(lbm::launch_fused_batch(b->mode, b->storage, b->cpt, b->d_ch[par], n, sc,
+                                           b->ntiles, b->d_counter, launch_grid(b), s));
 }
 
 int build_graph(lbm_batch *b) {
   drop_graph(b);
   LBM_CUDA(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
   int rc = LBM_OK;
-  for (int k = 0; k < b->chunk && rc == LBM_OK; k++) rc = launch_one(b, k, b->cap_stream);
+  for (int k = 0; k < b->chunk && rc == LBM_OK; k++) rc = launch_one(b, k, k & 1, b->cap_stream);
   cudaError_t e = cudaStreamEndCapture(b->cap_stream, &b->graph);
   if (rc != LBM_OK) return rc;
   LBM_CUDA(e);
@@ -261,6 +279,13 @@ int lbm_batch_create(lbm_h *lattices, int n, lbm_batch_h *out) {
     delete b;
     return cuda_fail(e);
   }
+  b->sweep_slots = lbm::sweep_batch_slots(b->mode, b->storage, b->device);
+  // 16-bit rounding turns the last-bit differences between the kernels into differences of
+  // the storage's precision, so such a batch takes the kernel that its lattices run alone
+  bool by_warps = true;
+  for (auto *h : b->lat) by_warps = by_warps && (h->tile.strips > 0 || h->sweep.strips > 0);
+  b->sweep = b->sweep_slots > 0 && (b->storage == LBM_STORAGE_F32 || by_warps);
+  if (b->sweep) b->tile_cols = lbm::sweep_batch_width();
   b->tile_rows = default_rows(b);
   layout(b);
   *out = b;
@@ -300,10 +325,7 @@ int lbm_batch_step(lbm_batch_h b, long nsteps, void *stream) {
     } else {
       for (int k = 0; k < m; k++) {
         // k-th step of this chunk runs with the table of its parity in the call
-        const int par = (phase + k) & 1;
-        rc = cuda_fail(lbm::launch_fused_batch(b->mode, b->storage, b->cpt, b->d_ch[par], n,
-                                               b->d_sc + (size_t)k * n, b->ntiles, b->d_counter,
-                                               launch_grid(b), s));
+        rc = launch_one(b, k, (phase + k) & 1, s);
         if (rc) return rc;
       }
     }
@@ -340,6 +362,7 @@ int lbm_batch_set_tiling(lbm_batch_h b, int rows, int cols, int cols_per_thread)
   if (b->grid_of[cols_per_thread] < 1) return LBM_ERR_ARG;
   if (cols > lbm::fused_batch_width(cols_per_thread)) return LBM_ERR_ARG;
   if (cols_per_thread == 2 && (cols & 1)) return LBM_ERR_ARG;
+  b->sweep = false;
   b->tile_rows = rows;
   b->tile_cols = cols;
   b->cpt = cols_per_thread;
@@ -351,7 +374,7 @@ int lbm_batch_tiling(lbm_batch_h b, int *rows, int *cols, int *cols_per_thread) 
   if (!b) return LBM_ERR_ARG;
   if (rows) *rows = b->tile_rows;
   if (cols) *cols = b->tile_cols;
-  if (cols_per_thread) *cols_per_thread = b->cpt;
+  if (cols_per_thread) *cols_per_thread = b->sweep ? 2 : b->cpt;
   return LBM_OK;
 }
 
@@ -372,6 +395,7 @@ int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, v
   Cand win{b->tile_rows, b->tile_cols, b->cpt};
   int rc = LBM_OK;
   auto time_one = [&](const Cand &c) -> int {
+    b->sweep = false;
     b->tile_rows = c.rows;
     b->tile_cols = c.cols;
     b->cpt = c.cpt;

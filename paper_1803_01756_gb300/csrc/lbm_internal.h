@@ -114,6 +114,29 @@ cudaError_t sweep_bf16_launch(const DevParams &p, const void *gs, void *gout, co
                               float *Tout, unsigned *status, const StepScalars *sc,
                               const StepScalars &val, const SweepTiling &tl, cudaStream_t s);
 
+// warp sweep over many lattices (lbm_sweep_batch.cu; energy equation and pseudopotential
+// only): one launch per update and kSweepBatch lattices, whose physics are its arguments
+constexpr int kSweepBatch = 48;
+struct SweepBatchItem {
+  const DevParams *p;
+  int chunks;  // row chunks of the lattice
+};
+// resident CTAs on this device (0: the modes have no such kernel, or failure)
+int sweep_batch_slots(const DevParams &mode, int storage, int device);
+// the n lattices of the device table ch (buffers and status words) with scalars sc
+cudaError_t launch_sweep_batch(int storage, const SweepBatchItem *items, int n,
+                               const BatchChannel *ch, const StepScalars *sc, cudaStream_t s);
+int sweep_batch_strips(int nx);  // warps across a lattice of nx columns
+int sweep_batch_cols(int nx);    // CTAs across
+int sweep_batch_width();         // output columns of a warp
+int sweep_batch_warps();         // warps of a CTA
+int sweep_batch_f16_slots(const DevParams &mode, int device);
+cudaError_t sweep_batch_f16_launch(const SweepBatchItem *items, int n, const BatchChannel *ch,
+                                   const StepScalars *sc, cudaStream_t s);
+int sweep_batch_bf16_slots(const DevParams &mode, int device);
+cudaError_t sweep_batch_bf16_launch(const SweepBatchItem *items, int n, const BatchChannel *ch,
+                                    const StepScalars *sc, cudaStream_t s);
+
 // tile kernel (lbm_tile.cu): one launch per update, a CTA per strip of 64 columns and row
 // chunk, with a warp for every row of a tile and its halo
 struct TileTiling {

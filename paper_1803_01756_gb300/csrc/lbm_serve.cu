@@ -99,6 +99,10 @@ void retire(lbm_server *s, const std::shared_ptr<Job> &j, int state) {
   s->cv.notify_all();
 }
 
+// A lattice this large fills the GPU alone and is stepped alone, with the single-lattice
+// kernel.
+constexpr long long kAloneNodes = 1LL << 20;
+
 // Move queued jobs into the active set while slots and the HBM budget allow
 // (first come, first served; a job that does not fit blocks the ones behind it).
 void admit(lbm_server *s) {
@@ -115,8 +119,16 @@ void admit(lbm_server *s) {
       j->state = LBM_JOB_RUNNING;
     }
     lbm_params_t p = j->p;
-    p.kernel = LBM_KERNEL_FUSED;
+    // batched jobs on the fused kernel; one that is stepped alone on the library's choice of
+    // fused kernel (a lattice that no fused kernel covers is refused either way)
+    const bool alone = (long long)j->nx * j->ny >= kAloneNodes;
+    p.kernel = alone ? LBM_KERNEL_AUTO : LBM_KERNEL_FUSED;
     int rc = lbm_create(j->nx, j->ny, &p, &j->lat);
+    if (rc == LBM_OK && j->lat->kernel != LBM_KERNEL_FUSED) {
+      lbm_destroy(j->lat);
+      j->lat = nullptr;
+      rc = LBM_ERR_ARG;
+    }
     if (rc == LBM_OK && !j->rho0.empty())
       rc = lbm_write_fields(j->lat, j->rho0.data(), nullptr, s->stream);
     j->rho0.clear();
@@ -140,11 +152,6 @@ void drop_group(lbm_server::Group &g) {
 // One scheduling round: every group of active jobs with equal modes advances by the
 // same number of steps in one batched launch per step; then every job's status word is
 // read with one synchronisation, and finished jobs are read back and freed.
-// A lattice this large fills the GPU alone (about 4 tiles of the fused kernel per SM) and
-// runs faster in the single-lattice kernel than in the batched one (69 against 102 us per
-// update on 4096 x 512), so it is stepped alone.
-constexpr long long kAloneNodes = 1LL << 20;
-
 void round(lbm_server *s) {
   std::map<int, std::vector<std::shared_ptr<Job>>> groups;
   std::vector<std::shared_ptr<Job>> alone;

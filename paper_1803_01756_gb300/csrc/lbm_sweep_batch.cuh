@@ -1,0 +1,103 @@
+// The warp sweep (lbm_sweep.cuh) over many lattices in one launch.
+//
+// The lattices' physics travel as kernel arguments, so that a CTA reads them through the
+// constant bank like the single-lattice kernel (the CTA-sweep batch kernel copies them to
+// shared memory, and its loop reads them from there); the buffers of the step come from the
+// batch's device table.  A CTA finds its lattice by its index, four adjacent strips of one
+// row chunk; the hardware hands the CTAs out in order, largest lattices first.
+// lbm_sweep_batch.cu, lbm_sweep_batch_f16.cu and lbm_sweep_batch_bf16.cu instantiate one
+// storage each.
+#pragma once
+
+#include "lbm_sweep_launch.cuh"
+
+namespace lbm {
+
+namespace {
+
+struct SweepBatchArgs {
+  struct Entry {
+    DevParams p;
+    SweepConsts k;
+    int begin;         // index of the lattice's first CTA
+    int cols, chunks;  // its CTAs across and along
+  };
+  int n;
+  Entry e[kSweepBatch];
+};
+static_assert(sizeof(SweepBatchArgs) <= 32764 - 64, "kernel arguments");
+
+template <bool YW, bool XO, class ST>
+__global__ void __launch_bounds__(SNT, SMIN)
+    k_sweep_batch(const __grid_constant__ SweepBatchArgs a, const BatchChannel *__restrict__ ch,
+                  const StepScalars *__restrict__ sc) {
+  const int b = (int)blockIdx.x;
+  int lo = 0, hi = a.n - 1;  // last lattice whose first CTA is b or before
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (a.e[mid].begin <= b) lo = mid;
+    else hi = mid - 1;
+  }
+  const SweepBatchArgs::Entry &e = a.e[lo];
+  const BatchChannel &c = ch[lo];
+  const StepScalars ssc = sc[lo];
+  const int local = b - e.begin, col = local % e.cols, chunk = local / e.cols;
+  const int Y0 = (int)(((long long)chunk * e.p.ny) / e.chunks);
+  const int ye = (int)(((long long)(chunk + 1) * e.p.ny) / e.chunks);
+  __shared__ float4 rings[SW][4 * 3 * 32];
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  Sweep<YW, XO, true, true, ST> s(e.p, e.k, static_cast<const typename ST::T *>(c.gs),
+                                  static_cast<typename ST::T *>(c.gout), c.Tin, c.Tout, ssc,
+                                  sweep_c0(col * SW + warp, true), Y0, ye, rings[warp]);
+  s.run(c.status);
+}
+
+template <class ST>
+using SweepBatchFn = void (*)(SweepBatchArgs, const BatchChannel *, const StepScalars *);
+
+template <class ST>
+SweepBatchFn<ST> sweep_batch_variant(const DevParams &p) {
+  static const SweepBatchFn<ST> table[4] = {
+      k_sweep_batch<false, false, ST>, k_sweep_batch<false, true, ST>,
+      k_sweep_batch<true, false, ST>, k_sweep_batch<true, true, ST>};
+  return table[(p.y_walls ? 2 : 0) | (p.x_open ? 1 : 0)];
+}
+
+template <class ST>
+int sweep_batch_slots_t(const DevParams &p, int device) {
+  int sms = 0, occ = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, sweep_batch_variant<ST>(p), SNT, 0) !=
+          cudaSuccess)
+    return 0;
+  return sms * occ;
+}
+
+template <class ST>
+cudaError_t sweep_batch_launch_t(const SweepBatchItem *items, int n, const BatchChannel *ch,
+                                 const StepScalars *sc, cudaStream_t s) {
+  for (int i0 = 0; i0 < n; i0 += kSweepBatch) {
+    SweepBatchArgs a;
+    a.n = std::min(kSweepBatch, n - i0);
+    long long ctas = 0;
+    for (int i = 0; i < a.n; i++) {
+      const SweepBatchItem &it = items[i0 + i];
+      SweepBatchArgs::Entry &e = a.e[i];
+      e.p = *it.p;
+      e.k = sweep_consts(*it.p);
+      e.begin = (int)ctas;
+      e.cols = sweep_cols(sweep_strips(it.p->nx, true));
+      e.chunks = it.chunks;
+      ctas += (long long)e.cols * e.chunks;
+    }
+    if (ctas < 1 || ctas > 2147483647LL) return cudaErrorInvalidConfiguration;
+    sweep_batch_variant<ST>(*items[0].p)<<<(unsigned)ctas, SNT, 0, s>>>(a, ch + i0, sc + i0);
+    const cudaError_t err = cudaGetLastError();
+    if (err != cudaSuccess) return err;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace
+
+}  // namespace lbm

@@ -179,6 +179,9 @@ def _stream_ptr(stream) -> int:
     if stream is None:
         try:
             import torch
+            if torch.cuda.is_initialized():
+                # the current stream's handle without a Stream object
+                return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
             if torch.cuda.is_available():
                 return torch.cuda.current_stream().cuda_stream
         except ImportError:

@@ -103,6 +103,22 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
   return makespan;
 }
 
+// The row steps of the tallest tile of the warp sweep at tile height H (a lattice's rows are
+// divided evenly), which is the launch where every CTA is resident; 0 where they are not.
+int one_wave(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, int H,
+             long long &ntiles) {
+  long long ctas = 0;
+  int tallest = 0;
+  ntiles = 0;
+  for (const lbm_lattice *h : order) {
+    const int rows = std::min(H, h->ny), chunks = (h->ny + rows - 1) / rows;
+    ctas += (long long)lbm::sweep_batch_cols(h->nx) * chunks;
+    ntiles += (long long)lbm::sweep_batch_strips(h->nx) * chunks;
+    tallest = std::max(tallest, (h->ny + chunks - 1) / chunks);
+  }
+  return ctas <= b->sweep_slots ? tallest + 10 : 0;
+}
+
 // Default tile height.  Each candidate of 128 .. 16 rows is scored by the makespan of its
 // greedy schedule and the shortest wins, the taller on a tie.  Measured on GB300 against
 // fixed heights, this picks the best or within 4 % of it on four shapes: 12 channels of
@@ -137,6 +153,22 @@ int default_rows(const lbm_batch *b) {
       best_tiles = n;
     }
   }
+  // In the warp sweep every fourth height from 24 to 256 rows competes too where it makes one
+  // wave: the tallest tile is then the launch (GB300, FP32, us per update: 16 channels of 2.9 M
+  // nodes 91.9 at 48 rows, 76.8 at 36; 30 of 4.1 M 121.4 at 64, 108.9 at 56; 20 channels 98.0 at
+  // 48, 91.1 at 44; FP16 storage 109.9 and 90.6, 140.7 and 127.8).  In several waves the
+  // schedule does not tell heights so close apart (40 channels of 6.3 M nodes 170.4 at 96 rows
+  // and 163.5 at 92 in one wave, 178.7 at 40 in two; 96 channels 432.9 at 64 and 435.2 at 52, both in several).
+  if (b->sweep)
+    for (int H = 256; H >= 24; H -= 4) {
+      long long n = 0;
+      const int cost = one_wave(b, order, H, n);
+      if (cost > 0 && cost < best_cost) {
+        best = H;
+        best_cost = cost;
+        best_tiles = n;
+      }
+    }
   if (best_tiles >= b->sms) return best;
   const int occ = std::max(1, std::min(4, (b->sweep ? b->sweep_slots : b->grid) / b->sms));
   const double *kStep = occ >= 4 ? kStep4 : kStep3;

@@ -235,12 +235,11 @@ int lbm_droplet_stats(const double *rho, int nx, int ny, double threshold, doubl
    thermal and multiphase switches and the storage, and that use the fused kernel or
    the two-pass path (LBM_KERNEL_AUTO gives one of the two);
    sizes and all other parameters may differ.  Each step is one launch over the tiles of
-   all lattices, largest lattices first: with the energy equation and the pseudopotential
-   by independent warps (one launch for every 48 lattices), each on a strip of 54 columns of
-   a row chunk; in the other modes, with a tiling of their own (lbm_batch_set_tiling) and
-   with 16-bit storage, unless every lattice is on the library's kernel choice, by resident
-   CTAs that take tiles from one work-list through an atomic counter.  The
-   batch borrows the lattices: they stay
+   all lattices, largest lattices first: by independent warps (one launch for every 48
+   lattices), each on a strip of 54 columns of a row chunk (60 without the energy
+   equation); with a tiling of their own (lbm_batch_set_tiling) and with 16-bit storage,
+   unless every lattice is on the library's kernel choice, by resident CTAs that take tiles
+   from one work-list through an atomic counter.  The batch borrows the lattices: they stay
    owned by the caller, must outlive the batch, and while batched should be advanced
    only through lbm_batch_step (their own t, buffers and status words advance).
    A lattice's fields after lbm_batch_step equal those after lbm_step alone. */

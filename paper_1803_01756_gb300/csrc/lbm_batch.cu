@@ -21,7 +21,7 @@ struct lbm_batch {
   int grid_of[3] = {0, 0, 0};      // resident CTAs with 1 and 2 columns per thread (0: none)
   // The warp sweep runs the batch until a tiling of the CTA kernel is asked for
   // (lbm_batch_set_tiling, lbm_batch_autotune): its tiles are a warp's strip of a row chunk.
-  int sweep_slots = 0;             // its resident CTAs (0: the modes have no such kernel)
+  int sweep_slots = 0;             // its resident CTAs
   bool sweep = false;
   std::vector<lbm::SweepBatchItem> items;
   int ntiles = 0, grid = 0, sms = 1;
@@ -46,7 +46,7 @@ using lbm_host::cuda_fail;
 
 int tiles_of(const lbm_batch *b, const lbm_lattice *h, int rows, int cols) {
   const int H = std::min(rows, h->ny);
-  if (b->sweep) return lbm::sweep_batch_strips(h->nx) * ((h->ny + H - 1) / H);
+  if (b->sweep) return lbm::sweep_batch_strips(h->dp) * ((h->ny + H - 1) / H);
   return ((h->nx + cols - 1) / cols) * ((h->ny + H - 1) / H);
 }
 
@@ -75,19 +75,20 @@ void layout(lbm_batch *b) {
 
 // Greedy list schedule of the work-list at tile height H over the resident CTAs (CTAs in
 // launch order, each taken by the first free slot, costing its row steps: H + 15, in the warp
-// sweep H + 10): returns the makespan in row steps and the number of tiles.
+// sweep H + 10, or H + 2 without the energy equation): returns the makespan in row steps and
+// the number of tiles.
 double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, int H,
                 long long &ntiles) {
   const int W = b->tile_cols;
   std::priority_queue<double, std::vector<double>, std::greater<double>> slots;
   const int resident = b->sweep ? b->sweep_slots : b->grid;
-  const double fill = b->sweep ? 10.0 : 15.0;
+  const double fill = b->sweep ? lbm::sweep_batch_fill(b->mode.thermal != 0) : 15.0;
   for (int k = 0; k < resident; k++) slots.push(0.0);
   double makespan = 0.0;
   ntiles = 0;
   for (const lbm_lattice *h : order) {
     const int rows = std::min(H, h->ny);
-    const int strips = b->sweep ? lbm::sweep_batch_cols(h->nx) : (h->nx + W - 1) / W;
+    const int strips = b->sweep ? lbm::sweep_batch_cols(h->dp) : (h->nx + W - 1) / W;
     for (int y0 = 0; y0 < h->ny; y0 += rows) {
       const double len = std::min(rows, h->ny - y0) + fill;
       for (int x = 0; x < strips; x++) {
@@ -98,7 +99,7 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
         ntiles++;
       }
     }
-    if (b->sweep) ntiles += (long long)(lbm::sweep_batch_strips(h->nx) - strips) * ((h->ny + rows - 1) / rows);
+    if (b->sweep) ntiles += (long long)(lbm::sweep_batch_strips(h->dp) - strips) * ((h->ny + rows - 1) / rows);
   }
   return makespan;
 }
@@ -112,11 +113,11 @@ int one_wave(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, 
   ntiles = 0;
   for (const lbm_lattice *h : order) {
     const int rows = std::min(H, h->ny), chunks = (h->ny + rows - 1) / rows;
-    ctas += (long long)lbm::sweep_batch_cols(h->nx) * chunks;
-    ntiles += (long long)lbm::sweep_batch_strips(h->nx) * chunks;
+    ctas += (long long)lbm::sweep_batch_cols(h->dp) * chunks;
+    ntiles += (long long)lbm::sweep_batch_strips(h->dp) * chunks;
     tallest = std::max(tallest, (h->ny + chunks - 1) / chunks);
   }
-  return ctas <= b->sweep_slots ? tallest + 10 : 0;
+  return ctas <= b->sweep_slots ? tallest + lbm::sweep_batch_fill(b->mode.thermal != 0) : 0;
 }
 
 // Default tile height.  Each candidate of 128 .. 16 rows is scored by the makespan of its
@@ -317,7 +318,7 @@ int lbm_batch_create(lbm_h *lattices, int n, lbm_batch_h *out) {
   bool by_warps = true;
   for (auto *h : b->lat) by_warps = by_warps && (h->tile.strips > 0 || h->sweep.strips > 0);
   b->sweep = b->sweep_slots > 0 && (b->storage == LBM_STORAGE_F32 || by_warps);
-  if (b->sweep) b->tile_cols = lbm::sweep_batch_width();
+  if (b->sweep) b->tile_cols = lbm::sweep_batch_width(b->mode.thermal != 0);
   b->tile_rows = default_rows(b);
   layout(b);
   *out = b;

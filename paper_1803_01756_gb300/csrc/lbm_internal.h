@@ -114,22 +114,23 @@ cudaError_t sweep_bf16_launch(const DevParams &p, const void *gs, void *gout, co
                               float *Tout, unsigned *status, const StepScalars *sc,
                               const StepScalars &val, const SweepTiling &tl, cudaStream_t s);
 
-// warp sweep over many lattices (lbm_sweep_batch.cu; energy equation and pseudopotential
-// only): one launch per update and kSweepBatch lattices, whose physics are its arguments
+// warp sweep over many lattices (lbm_sweep_batch.cu): one launch per update and kSweepBatch
+// lattices, whose physics are its arguments
 constexpr int kSweepBatch = 48;
 struct SweepBatchItem {
   const DevParams *p;
   int chunks;  // row chunks of the lattice
 };
-// resident CTAs on this device (0: the modes have no such kernel, or failure)
+// resident CTAs on this device (0 on failure)
 int sweep_batch_slots(const DevParams &mode, int storage, int device);
 // the n lattices of the device table ch (buffers and status words) with scalars sc
 cudaError_t launch_sweep_batch(int storage, const SweepBatchItem *items, int n,
                                const BatchChannel *ch, const StepScalars *sc, cudaStream_t s);
-int sweep_batch_strips(int nx);  // warps across a lattice of nx columns
-int sweep_batch_cols(int nx);    // CTAs across
-int sweep_batch_width();         // output columns of a warp
-int sweep_batch_warps();         // warps of a CTA
+int sweep_batch_strips(const DevParams &p);  // warps across the lattice
+int sweep_batch_cols(const DevParams &p);    // CTAs across
+int sweep_batch_width(bool thermal);         // output columns of a warp
+int sweep_batch_fill(bool thermal);          // rows swept beside a chunk's own
+int sweep_batch_warps();                     // warps of a CTA
 int sweep_batch_f16_slots(const DevParams &mode, int device);
 cudaError_t sweep_batch_f16_launch(const SweepBatchItem *items, int n, const BatchChannel *ch,
                                    const StepScalars *sc, cudaStream_t s);

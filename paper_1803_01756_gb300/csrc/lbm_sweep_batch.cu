@@ -4,7 +4,6 @@
 namespace lbm {
 
 int sweep_batch_slots(const DevParams &mode, int storage, int device) {
-  if (!mode.thermal || !mode.multiphase) return 0;
   return storage == STORAGE_BF16  ? sweep_batch_bf16_slots(mode, device)
          : storage == STORAGE_F16 ? sweep_batch_f16_slots(mode, device)
                                   : sweep_batch_slots_t<StoreF32>(mode, device);
@@ -19,9 +18,10 @@ cudaError_t launch_sweep_batch(int storage, const SweepBatchItem *items, int n,
   }
 }
 
-int sweep_batch_strips(int nx) { return sweep_strips(nx, true); }
-int sweep_batch_cols(int nx) { return sweep_cols(sweep_strips(nx, true)); }
-int sweep_batch_width() { return sweep_width(true); }
+int sweep_batch_strips(const DevParams &p) { return sweep_strips(p.nx, p.thermal != 0); }
+int sweep_batch_cols(const DevParams &p) { return sweep_cols(sweep_batch_strips(p)); }
+int sweep_batch_width(bool thermal) { return sweep_width(thermal); }
+int sweep_batch_fill(bool thermal) { return 2 * sweep_rows(thermal); }
 int sweep_batch_warps() { return SW; }
 
 }  // namespace lbm

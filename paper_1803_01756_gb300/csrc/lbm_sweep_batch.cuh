@@ -27,7 +27,7 @@ struct SweepBatchArgs {
 };
 static_assert(sizeof(SweepBatchArgs) <= 32764 - 64, "kernel arguments");
 
-template <bool YW, bool XO, class ST>
+template <bool YW, bool XO, bool TH, bool MP, class ST>
 __global__ void __launch_bounds__(SNT, SMIN)
     k_sweep_batch(const __grid_constant__ SweepBatchArgs a, const BatchChannel *__restrict__ ch,
                   const StepScalars *__restrict__ sc) {
@@ -44,11 +44,11 @@ __global__ void __launch_bounds__(SNT, SMIN)
   const int local = b - e.begin, col = local % e.cols, chunk = local / e.cols;
   const int Y0 = (int)(((long long)chunk * e.p.ny) / e.chunks);
   const int ye = (int)(((long long)(chunk + 1) * e.p.ny) / e.chunks);
-  __shared__ float4 rings[SW][4 * 3 * 32];
+  __shared__ float4 rings[SW][TH ? 4 * 3 * 32 : 32];
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
-  Sweep<YW, XO, true, true, ST> s(e.p, e.k, static_cast<const typename ST::T *>(c.gs),
-                                  static_cast<typename ST::T *>(c.gout), c.Tin, c.Tout, ssc,
-                                  sweep_c0(col * SW + warp, true), Y0, ye, rings[warp]);
+  Sweep<YW, XO, TH, MP, ST> s(e.p, e.k, static_cast<const typename ST::T *>(c.gs),
+                              static_cast<typename ST::T *>(c.gout), c.Tin, c.Tout, ssc,
+                              sweep_c0(col * SW + warp, TH), Y0, ye, rings[warp]);
   s.run(c.status);
 }
 
@@ -57,10 +57,18 @@ using SweepBatchFn = void (*)(SweepBatchArgs, const BatchChannel *, const StepSc
 
 template <class ST>
 SweepBatchFn<ST> sweep_batch_variant(const DevParams &p) {
-  static const SweepBatchFn<ST> table[4] = {
-      k_sweep_batch<false, false, ST>, k_sweep_batch<false, true, ST>,
-      k_sweep_batch<true, false, ST>, k_sweep_batch<true, true, ST>};
-  return table[(p.y_walls ? 2 : 0) | (p.x_open ? 1 : 0)];
+#define KB(a, b, c, d) k_sweep_batch<a, b, c, d, ST>
+  static const SweepBatchFn<ST> table[16] = {
+      KB(false, false, false, false), KB(false, false, false, true), KB(false, false, true, false),
+      KB(false, false, true, true),   KB(false, true, false, false), KB(false, true, false, true),
+      KB(false, true, true, false),   KB(false, true, true, true),   KB(true, false, false, false),
+      KB(true, false, false, true),   KB(true, false, true, false),  KB(true, false, true, true),
+      KB(true, true, false, false),   KB(true, true, false, true),   KB(true, true, true, false),
+      KB(true, true, true, true)};
+#undef KB
+  const int k = (p.y_walls ? 8 : 0) | (p.x_open ? 4 : 0) | (p.thermal ? 2 : 0) |
+                (p.multiphase ? 1 : 0);
+  return table[k];
 }
 
 template <class ST>
@@ -86,7 +94,7 @@ cudaError_t sweep_batch_launch_t(const SweepBatchItem *items, int n, const Batch
       e.p = *it.p;
       e.k = sweep_consts(*it.p);
       e.begin = (int)ctas;
-      e.cols = sweep_cols(sweep_strips(it.p->nx, true));
+      e.cols = sweep_cols(sweep_strips(it.p->nx, it.p->thermal != 0));
       e.chunks = it.chunks;
       ctas += (long long)e.cols * e.chunks;
     }

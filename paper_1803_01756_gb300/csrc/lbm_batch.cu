@@ -88,18 +88,19 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
   ntiles = 0;
   for (const lbm_lattice *h : order) {
     const int rows = std::min(H, h->ny);
-    const int strips = b->sweep ? lbm::sweep_batch_cols(h->dp) : (h->nx + W - 1) / W;
-    for (int y0 = 0; y0 < h->ny; y0 += rows) {
-      const double len = std::min(rows, h->ny - y0) + fill;
-      for (int x = 0; x < strips; x++) {
+    const int chunks = (h->ny + rows - 1) / rows, strips = (h->nx + W - 1) / W;
+    long long done = 0;  // CTAs of the row chunks so far
+    for (int c = 0; c < chunks; c++) {
+      const double len = std::min(rows, h->ny - c * rows) + fill;
+      const long long upto = b->sweep ? lbm::sweep_batch_ctas(h->dp, c + 1) : done + strips;
+      for (; done < upto; done++) {
         const double t = slots.top() + len;
         slots.pop();
         slots.push(t);
         makespan = std::max(makespan, t);
-        ntiles++;
       }
     }
-    if (b->sweep) ntiles += (long long)(lbm::sweep_batch_strips(h->dp) - strips) * ((h->ny + rows - 1) / rows);
+    ntiles += tiles_of(b, h, H, W);
   }
   return makespan;
 }
@@ -113,7 +114,7 @@ int one_wave(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, 
   ntiles = 0;
   for (const lbm_lattice *h : order) {
     const int rows = std::min(H, h->ny), chunks = (h->ny + rows - 1) / rows;
-    ctas += (long long)lbm::sweep_batch_cols(h->dp) * chunks;
+    ctas += lbm::sweep_batch_ctas(h->dp, chunks);
     ntiles += (long long)lbm::sweep_batch_strips(h->dp) * chunks;
     tallest = std::max(tallest, (h->ny + chunks - 1) / chunks);
   }

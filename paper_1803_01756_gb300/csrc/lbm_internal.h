@@ -127,7 +127,7 @@ int sweep_batch_slots(const DevParams &mode, int storage, int device);
 cudaError_t launch_sweep_batch(int storage, const SweepBatchItem *items, int n,
                                const BatchChannel *ch, const StepScalars *sc, cudaStream_t s);
 int sweep_batch_strips(const DevParams &p);  // warps across the lattice
-int sweep_batch_cols(const DevParams &p);    // CTAs across
+long long sweep_batch_ctas(const DevParams &p, int chunks);  // its CTAs with that many row chunks
 int sweep_batch_width(bool thermal);         // output columns of a warp
 int sweep_batch_fill(bool thermal);          // rows swept beside a chunk's own
 int sweep_batch_warps();                     // warps of a CTA

@@ -21,21 +21,22 @@ SweepTiling sweep_tiling(const DevParams &p, int storage, int device) {
   // from the shorter row step than they lose (GB300, FP32, us per update by row chunks:
   // 4096 x 512 47.9 at 24, 69 at 14; 2048 x 512 30.5 at 45, 37.2 at 32, 46.3 at 23;
   // 1237 x 531 23.3 at 76, 25.0 at 48, 27.9 at 38; 777 x 333 17.4 at 114 and at 66).
-  const int cols = sweep_cols(tl.strips), slots = sms * occ;
+  const long long slots = (long long)sms * occ;
   const int fill = 2 * sweep_rows(th);
   long long best = -1;
-  for (long long c = 1; c <= p.ny && (c - 1) * cols <= 3LL * slots; c++) {
-    const long long waves = (cols * c + slots - 1) / slots;
+  for (int c = 1; c <= p.ny && sweep_ctas(tl.strips, c - 1) <= 3 * slots; c++) {
+    const long long waves = (sweep_ctas(tl.strips, c) + slots - 1) / slots;
     const long long cost = waves * ((p.ny + c - 1) / c + fill);
     if (best < 0 || cost < best) {
       best = cost;
-      tl.chunks = (int)c;
+      tl.chunks = c;
     }
   }
   // Programmatic dependent launch when the grid fills at least 90 % of the wave, as for the
   // CTA sweep: below that the waiting CTAs of the next update take issue slots (2048 x 512 at
   // 23 chunks: 46.3 against 39.4 us per update; at 45 chunks 30.5 either way).
-  tl.pdl = cols * tl.chunks * 10 >= slots * 9 && cols * tl.chunks <= slots ? 1 : 0;
+  const long long ctas = sweep_ctas(tl.strips, tl.chunks);
+  tl.pdl = ctas * 10 >= slots * 9 && ctas <= slots ? 1 : 0;
   return tl;
 }
 

@@ -19,7 +19,9 @@ cudaError_t launch_sweep_batch(int storage, const SweepBatchItem *items, int n,
 }
 
 int sweep_batch_strips(const DevParams &p) { return sweep_strips(p.nx, p.thermal != 0); }
-int sweep_batch_cols(const DevParams &p) { return sweep_cols(sweep_batch_strips(p)); }
+long long sweep_batch_ctas(const DevParams &p, int chunks) {
+  return sweep_ctas(sweep_batch_strips(p), chunks);
+}
 int sweep_batch_width(bool thermal) { return sweep_width(thermal); }
 int sweep_batch_fill(bool thermal) { return 2 * sweep_rows(thermal); }
 int sweep_batch_warps() { return SW; }

@@ -3,8 +3,9 @@
 // The lattices' physics travel as kernel arguments, so that a CTA reads them through the
 // constant bank like the single-lattice kernel (the CTA-sweep batch kernel copies them to
 // shared memory, and its loop reads them from there); the buffers of the step come from the
-// batch's device table.  A CTA finds its lattice by its index, four adjacent strips of one
-// row chunk; the hardware hands the CTAs out in order, largest lattices first.
+// batch's device table.  A CTA finds its lattice by its index; its warps take the
+// lattice's tiles as in the single-lattice kernel, and the hardware hands the CTAs out in order, largest
+// lattices first.
 // lbm_sweep_batch.cu, lbm_sweep_batch_f16.cu and lbm_sweep_batch_bf16.cu instantiate one
 // storage each.
 #pragma once
@@ -20,7 +21,7 @@ struct SweepBatchArgs {
     DevParams p;
     SweepConsts k;
     int begin;         // index of the lattice's first CTA
-    int cols, chunks;  // its CTAs across and along
+    int strips, chunks;
   };
   int n;
   Entry e[kSweepBatch];
@@ -41,14 +42,17 @@ __global__ void __launch_bounds__(SNT, SMIN)
   const SweepBatchArgs::Entry &e = a.e[lo];
   const BatchChannel &c = ch[lo];
   const StepScalars ssc = sc[lo];
-  const int local = b - e.begin, col = local % e.cols, chunk = local / e.cols;
-  const int Y0 = (int)(((long long)chunk * e.p.ny) / e.chunks);
-  const int ye = (int)(((long long)(chunk + 1) * e.p.ny) / e.chunks);
   __shared__ float4 rings[SW][TH ? 4 * 3 * 32 : 32];
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+  const int cols = sweep_cols(e.strips), local = b - e.begin;
+  const SweepTile t =
+      sweep_tile<sweep_div<YW, XO, ST>()>(e.strips, local % cols, local / cols, warp);
+  if (t.chunk >= e.chunks) return;
+  const int Y0 = (int)(((long long)t.chunk * e.p.ny) / e.chunks);
+  const int ye = (int)(((long long)(t.chunk + 1) * e.p.ny) / e.chunks);
   Sweep<YW, XO, TH, MP, ST> s(e.p, e.k, static_cast<const typename ST::T *>(c.gs),
                               static_cast<typename ST::T *>(c.gout), c.Tin, c.Tout, ssc,
-                              sweep_c0(col * SW + warp, TH), Y0, ye, rings[warp]);
+                              sweep_c0(t.strip, TH), Y0, ye, rings[warp]);
   s.run(c.status);
 }
 
@@ -94,9 +98,9 @@ cudaError_t sweep_batch_launch_t(const SweepBatchItem *items, int n, const Batch
       e.p = *it.p;
       e.k = sweep_consts(*it.p);
       e.begin = (int)ctas;
-      e.cols = sweep_cols(sweep_strips(it.p->nx, it.p->thermal != 0));
+      e.strips = sweep_strips(it.p->nx, it.p->thermal != 0);
       e.chunks = it.chunks;
-      ctas += (long long)e.cols * e.chunks;
+      ctas += sweep_ctas(e.strips, e.chunks);
     }
     if (ctas < 1 || ctas > 2147483647LL) return cudaErrorInvalidConfiguration;
     sweep_batch_variant<ST>(*items[0].p)<<<(unsigned)ctas, SNT, 0, s>>>(a, ch + i0, sc + i0);

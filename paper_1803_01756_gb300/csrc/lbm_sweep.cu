@@ -15,19 +15,24 @@ SweepTiling sweep_tiling(const DevParams &p, int storage, int device) {
   const bool th = p.thermal != 0;
   tl.strips = sweep_strips(p.nx, th);
   tl.width = sweep_width(th);
-  // The fewest row steps: a wave of resident CTAs with chunks of H rows takes H + 10 of them
-  // (H + 2 without the energy equation).  That is one wave with the shortest chunks, unless
-  // the strips alone nearly fill it: beside a full SM the fewer, taller chunks of a partly filled one gain less
-  // from the shorter row step than they lose (GB300, FP32, us per update by row chunks:
-  // 4096 x 512 47.9 at 24, 69 at 14; 2048 x 512 30.5 at 45, 37.2 at 32, 46.3 at 23;
-  // 1237 x 531 23.3 at 76, 25.0 at 48, 27.9 at 38; 777 x 333 17.4 at 114 and at 66).
+  // The shortest launch.  A warp with H rows sweeps H of them in full and the halo's row steps
+  // (10; 2 without the energy equation) for about four fifths, since the pipeline fills there,
+  // and a row step takes longer the more CTAs share the SM: 0.71, 0.86 and 1 of the full SM's
+  // for one, two and three.  Several waves take a full SM's time each.  GB300, FP32, us per
+  // update at one, two and three CTAs per SM: 1000 x 300 19.7, 16.5, 18.7; 520 x 510 20.5, 17.4,
+  // 18.7; 2048 x 256 28.4, 21.7, 21.7; 1237 x 531 32.8, 24.2, 23.2; 2048 x 512 46.6, 32.5, 30.9;
+  // 1300 x 900 57.2, 39.7, 36.6, at two waves 49; FP16 storage 1000 x 300 26.2, 20.3, 21.3;
+  // 1237 x 531 41.8, 29.2, 27.1; without the energy equation 1000 x 300 9.6, 7.3, 7.1;
+  // 1237 x 531 17.3, 11.6, 9.9.
   const long long slots = (long long)sms * occ;
-  const int fill = 2 * sweep_rows(th);
-  long long best = -1;
+  const double fill = 0.8 * 2 * sweep_rows(th);
+  double best = -1.0;
   for (int c = 1; c <= p.ny && sweep_ctas(tl.strips, c - 1) <= 3 * slots; c++) {
-    const long long waves = (sweep_ctas(tl.strips, c) + slots - 1) / slots;
-    const long long cost = waves * ((p.ny + c - 1) / c + fill);
-    if (best < 0 || cost < best) {
+    const long long ctas = sweep_ctas(tl.strips, c), waves = (ctas + slots - 1) / slots;
+    const long long per_sm = (ctas + sms - 1) / sms;
+    const double step = waves > 1 ? (double)waves : 0.57 + 0.43 * (double)per_sm / occ;
+    const double cost = step * ((p.ny + c - 1) / c + fill);
+    if (best < 0.0 || cost < best) {
       best = cost;
       tl.chunks = c;
     }

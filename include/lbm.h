@@ -230,19 +230,21 @@ typedef struct lbm_droplet_stats {
 int lbm_droplet_stats(const double *rho, int nx, int ny, double threshold, double rho_v,
                       int periodic_x, lbm_droplet_stats_t *out);
 
-/* ---- batched updates of many lattices (one persistent launch per step) ----
+/* ---- batched updates of many lattices (one launch per step) ----
    A batch groups lattices that share the boundary modes (x_bc class, y_bc), the
    thermal and multiphase switches and the storage, and that use the fused kernel or
    the two-pass path (LBM_KERNEL_AUTO gives one of the two);
    sizes and all other parameters may differ.  Each step is one launch over the tiles of
-   all lattices, largest lattices first: by independent warps (one launch for every 48
-   lattices), each on a strip of 54 columns of a row chunk (60 without the energy
-   equation); with a tiling of their own (lbm_batch_set_tiling) and with 16-bit storage,
-   unless every lattice is on the library's kernel choice, by resident CTAs that take tiles
-   from one work-list through an atomic counter.  The batch borrows the lattices: they stay
-   owned by the caller, must outlive the batch, and while batched should be advanced
-   only through lbm_batch_step (their own t, buffers and status words advance).
-   A lattice's fields after lbm_batch_step equal those after lbm_step alone. */
+   all lattices, largest lattices first: those on the library's kernel choice
+   (LBM_KERNEL_AUTO) by independent warps (one launch for every 48 lattices), each on a strip
+   of 54 columns of a row chunk (60 without the energy equation); those on a kernel that
+   the caller named, in a launch of their own where the batch holds both, by resident CTAs
+   that take tiles from one work-list through an atomic counter.  The batch borrows the
+   lattices: they stay owned by the caller, must outlive the batch, and while batched should
+   be advanced only through lbm_batch_step (their own t, buffers and status words advance).
+   A lattice's fields after lbm_batch_step equal those after lbm_step alone, in every
+   storage: bit for bit on the library's kernel choice, within the FP32 parity bound (1e-5)
+   on a named kernel. */
 typedef struct lbm_batch *lbm_batch_h;
 
 /* LBM_ERR_ARG if a lattice is NULL, repeated, on another device, on the split path, or
@@ -261,9 +263,10 @@ int lbm_batch_set_graph(lbm_batch_h b, int enable);
 int lbm_batch_set_tile_rows(lbm_batch_h b, int rows);
 /* Set the tiling: output rows and columns per tile and lattice columns per thread (1, or 2
    when the batch's modes include the energy equation and the pseudopotential forces; cols
-   at most 118 with one column per thread, an even number up to 244 with two) of the
-   work-list kernel, which runs the batch from then on.  LBM_ERR_ARG otherwise.  Results do
-   not depend on the tiling. */
+   at most 118 with one column per thread, an even number up to 244 with two).  LBM_ERR_ARG
+   otherwise.  Lattices on the library's kernel choice take the rows alone: a warp's strip has
+   its own width and two columns per thread, which lbm_batch_tiling gives for a batch of them.
+   Results do not depend on the tiling. */
 int lbm_batch_set_tiling(lbm_batch_h b, int rows, int cols, int cols_per_thread);
 int lbm_batch_tiling(lbm_batch_h b, int *rows, int *cols, int *cols_per_thread);
 /* The library's autotuner: times tilings with steps_per_candidate timed updates each (plus

@@ -1,4 +1,4 @@
-// Batched updates of many lattices in one persistent launch per step.
+// Batched updates of many lattices, one launch per step for those of a kernel.
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -14,17 +14,21 @@ struct lbm_batch {
   int device = 0;
   int storage = 0;
   lbm::DevParams mode{};  // boundary modes and physics switches shared by all lattices
-  std::vector<lbm_lattice *> lat;  // work-list order: most tiles first
+  // A lattice runs in the batch with the arithmetic it has alone, and so has the same bits: the
+  // first nsweep lattices (on the tile kernel or the warp sweep alone) in the batched warp
+  // sweep, whose tiles are a warp's strip of a row chunk, the others (on the CTA sweep or the
+  // two passes alone) in the work-list kernel.  In each part those with most tiles come first.
+  std::vector<lbm_lattice *> lat;
+  int nsweep = 0;
+  int sweep_rows = 64;             // output rows per tile of the warp sweep
+  int sweep_slots = 0;             // its resident CTAs
+  std::vector<lbm::SweepBatchItem> items;
   int tile_rows = 64;              // output rows per tile (default_rows, or set / autotuned)
   int tile_cols = 0;               // output columns per tile (even with two columns per thread)
-  int cpt = 1;                     // lattice columns per thread of the batched kernel
+  int cpt = 1;                     // lattice columns per thread of the work-list kernel
   int grid_of[3] = {0, 0, 0};      // resident CTAs with 1 and 2 columns per thread (0: none)
-  // The warp sweep runs the batch until a tiling of the CTA kernel is asked for
-  // (lbm_batch_set_tiling, lbm_batch_autotune): its tiles are a warp's strip of a row chunk.
-  int sweep_slots = 0;             // its resident CTAs
-  bool sweep = false;
-  std::vector<lbm::SweepBatchItem> items;
-  int ntiles = 0, grid = 0, sms = 1;
+  int ntiles = 0, grid = 0, sms = 1;  // of the work-list
+  int sweep_tiles = 0;
   BatchChannel *d_ch[2] = {nullptr, nullptr};  // tables for even and odd steps of a call
   std::vector<BatchChannel> h_ch[2];
   StepScalars *d_sc = nullptr;                  // [chunk][n] scalars of the next chunk
@@ -44,10 +48,12 @@ namespace {
 
 using lbm_host::cuda_fail;
 
-int tiles_of(const lbm_batch *b, const lbm_lattice *h, int rows, int cols) {
-  const int H = std::min(rows, h->ny);
-  if (b->sweep) return lbm::sweep_batch_strips(h->dp) * ((h->ny + H - 1) / H);
-  return ((h->nx + cols - 1) / cols) * ((h->ny + H - 1) / H);
+bool swept(const lbm_lattice *h) { return h->tile.strips > 0 || h->sweep.strips > 0; }
+
+int tiles_of(const lbm_batch *b, const lbm_lattice *h, int rows) {
+  const int H = std::min(rows, h->ny), chunks = (h->ny + H - 1) / H;
+  return (swept(h) ? lbm::sweep_batch_strips(h->dp) : (h->nx + b->tile_cols - 1) / b->tile_cols) *
+         chunks;
 }
 
 void drop_graph(lbm_batch *b) {
@@ -57,32 +63,39 @@ void drop_graph(lbm_batch *b) {
   b->graph = nullptr;
 }
 
-// Work-list layout for the current tile height: lattices with the most work first
+// Layout for the current tile heights: lattices with the most work first
 void layout(lbm_batch *b) {
+  auto work = [&](const lbm_lattice *h) {
+    return (long long)tiles_of(b, h, swept(h) ? b->sweep_rows : b->tile_rows) * h->nx;
+  };
   std::stable_sort(b->lat.begin(), b->lat.end(), [&](const lbm_lattice *x, const lbm_lattice *y) {
-    return (long long)tiles_of(b, x, b->tile_rows, b->tile_cols) * x->nx >
-           (long long)tiles_of(b, y, b->tile_rows, b->tile_cols) * y->nx;
+    return swept(x) != swept(y) ? swept(x) : work(x) > work(y);
   });
-  b->ntiles = 0;
-  for (auto *h : b->lat) b->ntiles += tiles_of(b, h, b->tile_rows, b->tile_cols);
-  b->grid = b->sweep ? b->sweep_slots * lbm::sweep_batch_warps() : b->grid_of[b->cpt];
   b->items.clear();
-  if (b->sweep)
-    for (auto *h : b->lat)
-      b->items.push_back({&h->dp, (h->ny + b->tile_rows - 1) / b->tile_rows});
+  b->sweep_tiles = b->ntiles = 0;
+  for (auto *h : b->lat) {
+    if (swept(h)) {
+      b->sweep_tiles += tiles_of(b, h, b->sweep_rows);
+      b->items.push_back({&h->dp, (h->ny + b->sweep_rows - 1) / b->sweep_rows});
+    } else {
+      b->ntiles += tiles_of(b, h, b->tile_rows);
+    }
+  }
+  b->grid = b->grid_of[b->cpt];
   drop_graph(b);
 }
 
-// Greedy list schedule of the work-list at tile height H over the resident CTAs (CTAs in
+// Greedy list schedule of lattices of one kernel at tile height H over the resident CTAs (CTAs in
 // launch order, each taken by the first free slot, costing its row steps: H + 15, in the warp
 // sweep H + 10, or H + 2 without the energy equation): returns the makespan in row steps and
 // the number of tiles.
 double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, int H,
                 long long &ntiles) {
   const int W = b->tile_cols;
+  const bool sweep = swept(order[0]);
   std::priority_queue<double, std::vector<double>, std::greater<double>> slots;
-  const int resident = b->sweep ? b->sweep_slots : b->grid;
-  const double fill = b->sweep ? lbm::sweep_batch_fill(b->mode.thermal != 0) : 15.0;
+  const int resident = sweep ? b->sweep_slots : b->grid_of[b->cpt];
+  const double fill = sweep ? lbm::sweep_batch_fill(b->mode.thermal != 0) : 15.0;
   for (int k = 0; k < resident; k++) slots.push(0.0);
   double makespan = 0.0;
   ntiles = 0;
@@ -92,7 +105,7 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
     long long done = 0;  // CTAs of the row chunks so far
     for (int c = 0; c < chunks; c++) {
       const double len = std::min(rows, h->ny - c * rows) + fill;
-      const long long upto = b->sweep ? lbm::sweep_batch_ctas(h->dp, c + 1) : done + strips;
+      const long long upto = sweep ? lbm::sweep_batch_ctas(h->dp, c + 1) : done + strips;
       for (; done < upto; done++) {
         const double t = slots.top() + len;
         slots.pop();
@@ -100,7 +113,7 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
         makespan = std::max(makespan, t);
       }
     }
-    ntiles += tiles_of(b, h, H, W);
+    ntiles += tiles_of(b, h, H);
   }
   return makespan;
 }
@@ -134,12 +147,15 @@ int one_wave(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, 
 // (200 x 50 alone: 1 row, 17.0 against 39.3 us per update with 16; 1024 x 128: 4 rows,
 // 22.8 against 39.6 us).  The figures are the CTA kernel's; the warp sweep is scheduled by
 // the same rule with its own row steps and CTAs.
-int default_rows(const lbm_batch *b) {
+int default_rows(const lbm_batch *b, bool sweep) {
   static const int tall[] = {128, 96, 64, 48, 32, 24, 16};
   static const int small[] = {16, 12, 8, 6, 4, 3, 2, 1};
   static const double kStep3[4] = {0.0, 0.85, 1.0, 1.15};
   static const double kStep4[5] = {0.0, 0.85, 0.97, 1.42, 1.64};
-  std::vector<const lbm_lattice *> order(b->lat.begin(), b->lat.end());
+  std::vector<const lbm_lattice *> order;
+  for (const lbm_lattice *h : b->lat)
+    if (swept(h) == sweep) order.push_back(h);
+  if (order.empty()) return 64;
   std::stable_sort(order.begin(), order.end(), [](const lbm_lattice *x, const lbm_lattice *y) {
     return (long long)x->nx * x->ny > (long long)y->nx * y->ny;
   });
@@ -161,7 +177,7 @@ int default_rows(const lbm_batch *b) {
   // 48, 91.1 at 44; FP16 storage 109.9 and 90.6, 140.7 and 127.8).  In several waves the
   // schedule does not tell heights so close apart (40 channels of 6.3 M nodes 170.4 at 96 rows
   // and 163.5 at 92 in one wave, 178.7 at 40 in two; 96 channels 432.9 at 64 and 435.2 at 52, both in several).
-  if (b->sweep)
+  if (sweep)
     for (int H = 256; H >= 24; H -= 4) {
       long long n = 0;
       const int cost = one_wave(b, order, H, n);
@@ -172,7 +188,7 @@ int default_rows(const lbm_batch *b) {
       }
     }
   if (best_tiles >= b->sms) return best;
-  const int occ = std::max(1, std::min(4, (b->sweep ? b->sweep_slots : b->grid) / b->sms));
+  const int occ = std::max(1, std::min(4, (sweep ? b->sweep_slots : b->grid_of[b->cpt]) / b->sms));
   const double *kStep = occ >= 4 ? kStep4 : kStep3;
   best_cost = 0.0;
   for (int H : small) {
@@ -212,7 +228,7 @@ int upload_tables(lbm_batch *b, cudaStream_t s) {
       c.strips = (h->nx + W - 1) / W;
       c.tile_begin = begin;
     }
-    begin += tiles_of(b, h, b->tile_rows, b->tile_cols);
+    if (!swept(h)) begin += tiles_of(b, h, b->tile_rows);
   }
   const size_t bytes = sizeof(BatchChannel) * b->lat.size();
   for (int par = 0; par < 2; par++)
@@ -220,16 +236,18 @@ int upload_tables(lbm_batch *b, cudaStream_t s) {
   return LBM_OK;
 }
 
-// CTAs of one launch: the resident grid, or one per tile when there are fewer tiles
+// CTAs of a launch of the work-list kernel: the resident grid, or one per tile when there are
+// fewer tiles
 int launch_grid(const lbm_batch *b) { return std::min(b->grid, b->ntiles); }
 
 // step k of a chunk with the buffers of table par
 int launch_one(lbm_batch *b, int k, int par, cudaStream_t s) {
-  const int n = (int)b->lat.size();
+  const int n = (int)b->lat.size(), ns = b->nsweep;
+  const BatchChannel *ch = b->d_ch[par];
   const StepScalars *sc = b->d_sc + (size_t)k * n;
-  if (b->sweep)
-    return cuda_fail(lbm::launch_sweep_batch(b->storage, b->items.data(), n, b->d_ch[par], sc, s));
-  return cuda_fail(lbm::launch_fused_batch(b->mode, b->storage, b->cpt, b->d_ch[par], n, sc,
+  if (ns > 0) LBM_CUDA(lbm::launch_sweep_batch(b->storage, b->items.data(), ns, ch, sc, s));
+  if (ns == n) return LBM_OK;
+  return cuda_fail(lbm::launch_fused_batch(b->mode, b->storage, b->cpt, ch + ns, n - ns, sc + ns,
                                            b->ntiles, b->d_counter, launch_grid(b), s));
 }
 
@@ -314,13 +332,14 @@ int lbm_batch_create(lbm_h *lattices, int n, lbm_batch_h *out) {
     return cuda_fail(e);
   }
   b->sweep_slots = lbm::sweep_batch_slots(b->mode, b->storage, b->device);
-  // 16-bit rounding turns the last-bit differences between the kernels into differences of
-  // the storage's precision, so such a batch takes the kernel that its lattices run alone
-  bool by_warps = true;
-  for (auto *h : b->lat) by_warps = by_warps && (h->tile.strips > 0 || h->sweep.strips > 0);
-  b->sweep = b->sweep_slots > 0 && (b->storage == LBM_STORAGE_F32 || by_warps);
-  if (b->sweep) b->tile_cols = lbm::sweep_batch_width(b->mode.thermal != 0);
-  b->tile_rows = default_rows(b);
+  for (auto *h : b->lat) b->nsweep += swept(h) ? 1 : 0;
+  if (b->nsweep > 0 && b->sweep_slots < 1) {
+    free_batch(b);
+    delete b;
+    return LBM_ERR_CUDA;
+  }
+  b->sweep_rows = default_rows(b, true);
+  b->tile_rows = default_rows(b, false);
   layout(b);
   *out = b;
   return LBM_OK;
@@ -385,7 +404,7 @@ int lbm_batch_set_graph(lbm_batch_h b, int enable) {
 
 int lbm_batch_set_tile_rows(lbm_batch_h b, int rows) {
   if (!b || rows < 1) return LBM_ERR_ARG;
-  b->tile_rows = rows;
+  b->sweep_rows = b->tile_rows = rows;
   layout(b);
   return LBM_OK;
 }
@@ -396,8 +415,8 @@ int lbm_batch_set_tiling(lbm_batch_h b, int rows, int cols, int cols_per_thread)
   if (b->grid_of[cols_per_thread] < 1) return LBM_ERR_ARG;
   if (cols > lbm::fused_batch_width(cols_per_thread)) return LBM_ERR_ARG;
   if (cols_per_thread == 2 && (cols & 1)) return LBM_ERR_ARG;
-  b->sweep = false;
-  b->tile_rows = rows;
+  // (the warp sweep takes the rows: its strips have their own width and two columns per lane)
+  b->sweep_rows = b->tile_rows = rows;
   b->tile_cols = cols;
   b->cpt = cols_per_thread;
   layout(b);
@@ -406,9 +425,10 @@ int lbm_batch_set_tiling(lbm_batch_h b, int rows, int cols, int cols_per_thread)
 
 int lbm_batch_tiling(lbm_batch_h b, int *rows, int *cols, int *cols_per_thread) {
   if (!b) return LBM_ERR_ARG;
-  if (rows) *rows = b->tile_rows;
-  if (cols) *cols = b->tile_cols;
-  if (cols_per_thread) *cols_per_thread = b->sweep ? 2 : b->cpt;
+  const bool all = b->nsweep == (int)b->lat.size();
+  if (rows) *rows = all ? b->sweep_rows : b->tile_rows;
+  if (cols) *cols = all ? lbm::sweep_batch_width(b->mode.thermal != 0) : b->tile_cols;
+  if (cols_per_thread) *cols_per_thread = all ? 2 : b->cpt;
   return LBM_OK;
 }
 
@@ -429,8 +449,7 @@ int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, v
   Cand win{b->tile_rows, b->tile_cols, b->cpt};
   int rc = LBM_OK;
   auto time_one = [&](const Cand &c) -> int {
-    b->sweep = false;
-    b->tile_rows = c.rows;
+    b->sweep_rows = b->tile_rows = c.rows;
     b->tile_cols = c.cols;
     b->cpt = c.cpt;
     layout(b);
@@ -471,7 +490,7 @@ int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, v
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   b->use_graph = graph;
-  b->tile_rows = win.rows;
+  b->sweep_rows = b->tile_rows = win.rows;
   b->tile_cols = win.cols;
   b->cpt = win.cpt;
   layout(b);
@@ -481,9 +500,11 @@ int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, v
 
 int lbm_batch_info(lbm_batch_h b, int *ntiles, int *grid, int *tile_rows) {
   if (!b) return LBM_ERR_ARG;
-  if (ntiles) *ntiles = b->ntiles;
-  if (grid) *grid = b->grid;
-  if (tile_rows) *tile_rows = b->tile_rows;
+  if (ntiles) *ntiles = b->sweep_tiles + b->ntiles;
+  if (grid)
+    *grid = (b->nsweep > 0 ? b->sweep_slots * lbm::sweep_batch_warps() : 0) +
+            (b->nsweep < (int)b->lat.size() ? b->grid : 0);
+  if (tile_rows) *tile_rows = b->nsweep == (int)b->lat.size() ? b->sweep_rows : b->tile_rows;
   return LBM_OK;
 }
 

@@ -273,10 +273,12 @@ int lbm_batch_tiling(lbm_batch_h b, int *rows, int *cols, int *cols_per_thread);
    two warm-up updates) and keeps the fastest.  Candidates: tile heights 16, 24, 32, 48, 64,
    96 and 128 rows at the widest tiles, for one column per thread and, where the modes allow
    it, two; then tiles of three quarters and half that width at the winner's height and
-   column count.  These are real updates: every lattice advances by
-   (7 k + 2) * (steps_per_candidate + 2) steps, k the number of column counts tried (1 or 2).
-   Writes the winning height to *best_rows (may be NULL; lbm_batch_tiling gives all three).
-   Synchronises the stream. */
+   column count.  A batch that is all on the library's kernel choice has one column count:
+   those heights, then the height in place and three quarters of the winner's.  These are real
+   updates: every lattice advances by (7 k + 2) * (steps_per_candidate + 2) steps, k the number
+   of column counts tried (1 or 2).  Writes the winning height to *best_rows (may be NULL;
+   lbm_batch_tiling gives all three).  On an error the tiling stays as it was.  Synchronises
+   the stream. */
 int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, void *stream);
 int lbm_batch_info(lbm_batch_h b, int *ntiles, int *grid, int *tile_rows);
 /* Synchronises the device, frees the batch's tables; the lattices are untouched. */

@@ -437,7 +437,7 @@ int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, v
   LBM_CUDA(cudaSetDevice(b->device));
   cudaStream_t s = (cudaStream_t)stream;
   struct Cand {
-    int rows, cols, cpt;
+    int sweep_rows, rows, cols, cpt;
   };
   static const int heights[] = {16, 24, 32, 48, 64, 96, 128};
   cudaEvent_t e0, e1;
@@ -446,13 +446,18 @@ int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, v
   const bool graph = b->use_graph;
   b->use_graph = false;
   float best = -1.0f;
-  Cand win{b->tile_rows, b->tile_cols, b->cpt};
+  const Cand before{b->sweep_rows, b->tile_rows, b->tile_cols, b->cpt};
+  Cand win = before;
   int rc = LBM_OK;
-  auto time_one = [&](const Cand &c) -> int {
-    b->sweep_rows = b->tile_rows = c.rows;
+  auto use = [&](const Cand &c) {
+    b->sweep_rows = c.sweep_rows;
+    b->tile_rows = c.rows;
     b->tile_cols = c.cols;
     b->cpt = c.cpt;
     layout(b);
+  };
+  auto time_one = [&](const Cand &c) -> int {
+    use(c);
     int r = lbm_batch_step(b, 2, stream);  // warm-up
     if (r) return r;
     LBM_CUDA(cudaEventRecord(e0, s));
@@ -468,33 +473,39 @@ int lbm_batch_autotune(lbm_batch_h b, int steps_per_candidate, int *best_rows, v
     }
     return LBM_OK;
   };
-  // tile heights at the widest tiles, for each column count the mode has a kernel for
-  for (int cpt = 1; cpt <= 2 && rc == LBM_OK; cpt++) {
-    if (b->grid_of[cpt] < 1) continue;
-    for (int H : heights) {
-      rc = time_one(Cand{H, lbm::fused_batch_width(cpt), cpt});
-      if (rc) break;
+  const bool all = b->nsweep == (int)b->lat.size();
+  if (all) {
+    // the warp sweep: the same heights, the height in place (the default lies between them where
+    // that makes one wave) and three quarters of the winner's
+    auto rows_only = [&](int H) { return Cand{H, H, before.cols, before.cpt}; };
+    for (int H : heights)
+      if (rc == LBM_OK) rc = time_one(rows_only(H));
+    if (rc == LBM_OK) rc = time_one(before);
+    if (rc == LBM_OK) rc = time_one(rows_only(std::max(1, win.sweep_rows * 3 / 4)));
+  } else {
+    // tile heights at the widest tiles, for each column count the mode has a kernel for
+    for (int cpt = 1; cpt <= 2 && rc == LBM_OK; cpt++) {
+      if (b->grid_of[cpt] < 1) continue;
+      for (int H : heights) {
+        rc = time_one(Cand{H, H, lbm::fused_batch_width(cpt), cpt});
+        if (rc) break;
+      }
     }
-  }
-  // then narrower tiles (three quarters and half the width) at the winner's height
-  if (rc == LBM_OK) {
+    // then narrower tiles (three quarters and half the width) at the winner's height
     const Cand base = win;
     const int Wmax = lbm::fused_batch_width(base.cpt);
     for (int num : {3, 2}) {
+      if (rc) break;
       int W = Wmax * num / 4;
       if (base.cpt == 2) W &= ~1;
-      rc = time_one(Cand{base.rows, W, base.cpt});
-      if (rc) break;
+      rc = time_one(Cand{base.sweep_rows, base.rows, W, base.cpt});
     }
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   b->use_graph = graph;
-  b->sweep_rows = b->tile_rows = win.rows;
-  b->tile_cols = win.cols;
-  b->cpt = win.cpt;
-  layout(b);
-  if (best_rows) *best_rows = win.rows;
+  use(rc == LBM_OK ? win : before);
+  if (best_rows) *best_rows = all ? b->sweep_rows : b->tile_rows;
   return rc;
 }
 

@@ -296,8 +296,10 @@ void lbm_batch_destroy(lbm_batch_h b);
    job has fewer left); it reads every job's status word with one synchronisation, reads
    finished jobs' fields back to host memory and frees their device memory, which admits
    the next jobs.
-   A job's fields equal those of the same job run alone (lbm_step) within the FP32
-   parity bound. */
+   A job whose parameters leave the kernel to the library (LBM_KERNEL_AUTO) runs on the
+   library's choice, any other on the fused kernel (LBM_KERNEL_FUSED).  Its fields equal those
+   of the same job run alone (lbm_step) on that kernel within the FP32 parity bound, in every
+   storage. */
 #define LBM_JOB_QUEUED 0
 #define LBM_JOB_RUNNING 1
 #define LBM_JOB_DONE 2  /* other final states are negative LBM_ERR_* codes */

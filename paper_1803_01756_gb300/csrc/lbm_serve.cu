@@ -119,12 +119,12 @@ void admit(lbm_server *s) {
       j->state = LBM_JOB_RUNNING;
     }
     lbm_params_t p = j->p;
-    // batched jobs on the fused kernel; one that is stepped alone on the library's choice of
-    // fused kernel (a lattice that no fused kernel covers is refused either way)
-    const bool alone = (long long)j->nx * j->ny >= kAloneNodes;
-    p.kernel = alone ? LBM_KERNEL_AUTO : LBM_KERNEL_FUSED;
+    // the library's kernel choice where the job leaves it to the library, so that its fields are
+    // those of the lattice alone; the fused kernel otherwise (a lattice that a batch does not
+    // take is refused either way)
+    if (p.kernel != LBM_KERNEL_AUTO) p.kernel = LBM_KERNEL_FUSED;
     int rc = lbm_create(j->nx, j->ny, &p, &j->lat);
-    if (rc == LBM_OK && j->lat->kernel != LBM_KERNEL_FUSED) {
+    if (rc == LBM_OK && j->lat->kernel == LBM_KERNEL_SPLIT) {
       lbm_destroy(j->lat);
       j->lat = nullptr;
       rc = LBM_ERR_ARG;

@@ -416,7 +416,11 @@ class Server:
 
     def submit(self, nx: int, ny: int, params: dict, nsteps: int, rho0=None,
                storage: int = STORAGE_F32, rho_ref: float = 0.0) -> int:
-        p = make_params(params, kernel=KERNEL_FUSED, storage=storage, rho_ref=rho_ref)
+        """Queue a job.  FP32 jobs run on the library's kernel choice, as ``Lattice`` does by
+        default; 16-bit ones on the fused kernel, and equal ``Lattice(..., kernel=KERNEL_FUSED)``
+        (the rounding of 16-bit storage makes the two differ at its precision)."""
+        kernel = KERNEL_AUTO if storage == STORAGE_F32 else KERNEL_FUSED
+        p = make_params(params, kernel=kernel, storage=storage, rho_ref=rho_ref)
         r = None
         if rho0 is not None:
             r = np.ascontiguousarray(rho0, dtype=np.float64).reshape(ny, nx)

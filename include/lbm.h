@@ -236,7 +236,8 @@ int lbm_droplet_stats(const double *rho, int nx, int ny, double threshold, doubl
    the two-pass path (LBM_KERNEL_AUTO gives one of the two);
    sizes and all other parameters may differ.  Each step is one launch over the tiles of
    all lattices, largest lattices first: those on the library's kernel choice
-   (LBM_KERNEL_AUTO) by independent warps (one launch for every 48 lattices), each on a strip
+   (LBM_KERNEL_AUTO) by independent warps (one launch for every 48 lattices, the launches
+   beside one another on streams of the batch), each on a strip
    of 54 columns of a row chunk (60 without the energy equation); those on a kernel that
    the caller named, in a launch of their own where the batch holds both, by resident CTAs
    that take tiles from one work-list through an atomic counter.  The batch borrows the

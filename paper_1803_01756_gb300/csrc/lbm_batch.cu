@@ -29,6 +29,19 @@ struct lbm_batch {
   int grid_of[3] = {0, 0, 0};      // resident CTAs with 1 and 2 columns per thread (0: none)
   int ntiles = 0, grid = 0, sms = 1;  // of the work-list
   int sweep_tiles = 0;
+  // The lattices of one launch, first .. first + n - 1 of lat: a launch of the warp sweep takes
+  // kSweepBatch of them at most, and the work-list kernel takes its own.  The lattices of
+  // different groups have nothing to do with one another, so each group runs its updates on a
+  // stream of its own and the GPU fills with all of them (192 channels of 100 x 32 at 8 rows:
+  // 34 us per update, 85 with the launches one after another).
+  struct Group {
+    bool sweep;
+    int first, n;
+    cudaStream_t stream;  // (the first group runs on the caller's)
+    cudaEvent_t done;
+  };
+  std::vector<Group> groups;
+  cudaEvent_t fork = nullptr;
   BatchChannel *d_ch[2] = {nullptr, nullptr};  // tables for even and odd steps of a call
   std::vector<BatchChannel> h_ch[2];
   StepScalars *d_sc = nullptr;                  // [chunk][n] scalars of the next chunk
@@ -71,6 +84,15 @@ void layout(lbm_batch *b) {
   std::stable_sort(b->lat.begin(), b->lat.end(), [&](const lbm_lattice *x, const lbm_lattice *y) {
     return swept(x) != swept(y) ? swept(x) : work(x) > work(y);
   });
+  // each group of the sweep gets its share of the large lattices and of the small ones
+  const std::vector<lbm_lattice *> sorted = b->lat;
+  const int ng = (b->nsweep + lbm::kSweepBatch - 1) / lbm::kSweepBatch;
+  int at = 0;
+  for (int g = 0; g < ng; g++) {
+    b->groups[g].first = at;
+    for (int i = g; i < b->nsweep; i += ng) b->lat[at++] = sorted[i];
+    b->groups[g].n = at - b->groups[g].first;
+  }
   b->items.clear();
   b->sweep_tiles = b->ntiles = 0;
   for (auto *h : b->lat) {
@@ -83,6 +105,22 @@ void layout(lbm_batch *b) {
   }
   b->grid = b->grid_of[b->cpt];
   drop_graph(b);
+}
+
+// the groups, their streams and events
+cudaError_t make_groups(lbm_batch *b) {
+  const int n = (int)b->lat.size();
+  for (int at = 0; at < b->nsweep; at += lbm::kSweepBatch)
+    b->groups.push_back({true, 0, 0, nullptr, nullptr});
+  if (b->nsweep < n) b->groups.push_back({false, b->nsweep, n - b->nsweep, nullptr, nullptr});
+  cudaError_t e = cudaSuccess;
+  for (size_t g = 1; g < b->groups.size() && e == cudaSuccess; g++) {
+    e = cudaStreamCreateWithFlags(&b->groups[g].stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->groups[g].done, cudaEventDisableTiming);
+  }
+  if (b->groups.size() > 1 && e == cudaSuccess)
+    e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+  return e;
 }
 
 // Greedy list schedule of lattices of one kernel at tile height H over the resident CTAs (CTAs in
@@ -240,22 +278,39 @@ int upload_tables(lbm_batch *b, cudaStream_t s) {
 // fewer tiles
 int launch_grid(const lbm_batch *b) { return std::min(b->grid, b->ntiles); }
 
-// step k of a chunk with the buffers of table par
-int launch_one(lbm_batch *b, int k, int par, cudaStream_t s) {
-  const int n = (int)b->lat.size(), ns = b->nsweep;
-  const BatchChannel *ch = b->d_ch[par];
-  const StepScalars *sc = b->d_sc + (size_t)k * n;
-  if (ns > 0) LBM_CUDA(lbm::launch_sweep_batch(b->storage, b->items.data(), ns, ch, sc, s));
-  if (ns == n) return LBM_OK;
-  return cuda_fail(lbm::launch_fused_batch(b->mode, b->storage, b->cpt, ch + ns, n - ns, sc + ns,
-                                           b->ntiles, b->d_counter, launch_grid(b), s));
+// step k of a chunk of group g with the buffers of table par
+cudaError_t launch_one(lbm_batch *b, const lbm_batch::Group &g, int k, int par, cudaStream_t s) {
+  const BatchChannel *ch = b->d_ch[par] + g.first;
+  const StepScalars *sc = b->d_sc + (size_t)k * b->lat.size() + g.first;
+  if (g.sweep) return lbm::launch_sweep_batch(b->storage, b->items.data() + g.first, g.n, ch, sc, s);
+  return lbm::launch_fused_batch(b->mode, b->storage, b->cpt, ch, g.n, sc, b->ntiles, b->d_counter,
+                                 launch_grid(b), s);
+}
+
+// The m steps of a chunk, the first with table phase: the groups beside one another, each on
+// its stream, behind the work of stream s and before what follows on it.
+int launch_chunk(lbm_batch *b, int m, int phase, cudaStream_t s) {
+  const int ng = (int)b->groups.size();
+  if (ng > 1) LBM_CUDA(cudaEventRecord(b->fork, s));
+  int forked = 1;
+  cudaError_t e = cudaSuccess;
+  for (; forked < ng && e == cudaSuccess; forked++)
+    e = cudaStreamWaitEvent(b->groups[forked].stream, b->fork, 0);
+  for (int k = 0; k < m && e == cudaSuccess; k++)
+    for (int g = 0; g < ng && e == cudaSuccess; g++)
+      e = launch_one(b, b->groups[g], k, (phase + k) & 1, g ? b->groups[g].stream : s);
+  for (int g = 1; g < forked; g++) {  // (joined also when a launch failed)
+    cudaError_t j = cudaEventRecord(b->groups[g].done, b->groups[g].stream);
+    if (j == cudaSuccess) j = cudaStreamWaitEvent(s, b->groups[g].done, 0);
+    if (e == cudaSuccess) e = j;
+  }
+  return cuda_fail(e);
 }
 
 int build_graph(lbm_batch *b) {
   drop_graph(b);
   LBM_CUDA(cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = LBM_OK;
-  for (int k = 0; k < b->chunk && rc == LBM_OK; k++) rc = launch_one(b, k, k & 1, b->cap_stream);
+  const int rc = launch_chunk(b, b->chunk, 0, b->cap_stream);
   cudaError_t e = cudaStreamEndCapture(b->cap_stream, &b->graph);
   if (rc != LBM_OK) return rc;
   LBM_CUDA(e);
@@ -265,6 +320,11 @@ int build_graph(lbm_batch *b) {
 
 void free_batch(lbm_batch *b) {
   drop_graph(b);
+  for (auto &g : b->groups) {
+    if (g.done) cudaEventDestroy(g.done);
+    if (g.stream) cudaStreamDestroy(g.stream);
+  }
+  if (b->fork) cudaEventDestroy(b->fork);
   cudaFree(b->d_ch[0]);
   cudaFree(b->d_ch[1]);
   cudaFree(b->d_sc);
@@ -333,10 +393,11 @@ int lbm_batch_create(lbm_h *lattices, int n, lbm_batch_h *out) {
   }
   b->sweep_slots = lbm::sweep_batch_slots(b->mode, b->storage, b->device);
   for (auto *h : b->lat) b->nsweep += swept(h) ? 1 : 0;
-  if (b->nsweep > 0 && b->sweep_slots < 1) {
+  e = b->nsweep > 0 && b->sweep_slots < 1 ? cudaErrorUnknown : make_groups(b);
+  if (e != cudaSuccess) {
     free_batch(b);
     delete b;
-    return LBM_ERR_CUDA;
+    return cuda_fail(e);
   }
   b->sweep_rows = default_rows(b, true);
   b->tile_rows = default_rows(b, false);
@@ -376,11 +437,9 @@ int lbm_batch_step(lbm_batch_h b, long nsteps, void *stream) {
       }
       LBM_CUDA(cudaGraphLaunch(b->gexec, s));
     } else {
-      for (int k = 0; k < m; k++) {
-        // k-th step of this chunk runs with the table of its parity in the call
-        rc = launch_one(b, k, (phase + k) & 1, s);
-        if (rc) return rc;
-      }
+      // (phase: a step runs with the table of its parity in the call)
+      rc = launch_chunk(b, m, phase, s);
+      if (rc) return rc;
     }
     phase = (phase + m) & 1;
     done += m;

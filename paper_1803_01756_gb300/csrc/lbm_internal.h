@@ -114,8 +114,8 @@ cudaError_t sweep_bf16_launch(const DevParams &p, const void *gs, void *gout, co
                               float *Tout, unsigned *status, const StepScalars *sc,
                               const StepScalars &val, const SweepTiling &tl, cudaStream_t s);
 
-// warp sweep over many lattices (lbm_sweep_batch.cu): one launch per update and kSweepBatch
-// lattices, whose physics are its arguments
+// warp sweep over many lattices (lbm_sweep_batch.cu): one launch per update of at most
+// kSweepBatch lattices, whose physics are its arguments
 constexpr int kSweepBatch = 48;
 struct SweepBatchItem {
   const DevParams *p;

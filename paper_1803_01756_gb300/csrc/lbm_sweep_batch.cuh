@@ -88,26 +88,22 @@ int sweep_batch_slots_t(const DevParams &p, int device) {
 template <class ST>
 cudaError_t sweep_batch_launch_t(const SweepBatchItem *items, int n, const BatchChannel *ch,
                                  const StepScalars *sc, cudaStream_t s) {
-  for (int i0 = 0; i0 < n; i0 += kSweepBatch) {
-    SweepBatchArgs a;
-    a.n = std::min(kSweepBatch, n - i0);
-    long long ctas = 0;
-    for (int i = 0; i < a.n; i++) {
-      const SweepBatchItem &it = items[i0 + i];
-      SweepBatchArgs::Entry &e = a.e[i];
-      e.p = *it.p;
-      e.k = sweep_consts(*it.p);
-      e.begin = (int)ctas;
-      e.strips = sweep_strips(it.p->nx, it.p->thermal != 0);
-      e.chunks = it.chunks;
-      ctas += sweep_ctas(e.strips, e.chunks);
-    }
-    if (ctas < 1 || ctas > 2147483647LL) return cudaErrorInvalidConfiguration;
-    sweep_batch_variant<ST>(*items[0].p)<<<(unsigned)ctas, SNT, 0, s>>>(a, ch + i0, sc + i0);
-    const cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return err;
+  if (n < 1 || n > kSweepBatch) return cudaErrorInvalidValue;
+  SweepBatchArgs a;
+  a.n = n;
+  long long ctas = 0;
+  for (int i = 0; i < n; i++) {
+    SweepBatchArgs::Entry &e = a.e[i];
+    e.p = *items[i].p;
+    e.k = sweep_consts(e.p);
+    e.begin = (int)ctas;
+    e.strips = sweep_strips(e.p.nx, e.p.thermal != 0);
+    e.chunks = items[i].chunks;
+    ctas += sweep_ctas(e.strips, e.chunks);
+    if (ctas > 2147483647LL) return cudaErrorInvalidConfiguration;
   }
-  return cudaSuccess;
+  sweep_batch_variant<ST>(*items[0].p)<<<(unsigned)ctas, SNT, 0, s>>>(a, ch, sc);
+  return cudaGetLastError();
 }
 
 }  // namespace

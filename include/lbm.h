@@ -257,10 +257,11 @@ int lbm_batch_step(lbm_batch_h b, long nsteps, void *stream);
 /* enable != 0: replay whole chunks of 16 steps from one captured CUDA graph. */
 int lbm_batch_set_graph(lbm_batch_h b, int enable);
 /* Output rows per tile (the work-list granularity).  The default, chosen at creation, is the
-   height among 128, 96, 64, 48, 32, 24 and 16 rows (by independent warps also the multiples
-   of 4 from 24 to 256 that make one wave) whose work-list a greedy schedule over
-   the resident CTAs finishes first; if that leaves fewer tiles than SMs, heights down to
-   1 row compete, with row steps slower the more tiles share an SM. */
+   height among 128, 96, 64, 48, 32, 24 and 16 rows whose work-list a greedy schedule over
+   the resident CTAs finishes first.  By independent warps the heights that make one wave of
+   CTAs compete by that wave's time (1 to 24 rows, and the multiples of 4 up to 256); by the
+   work-list kernel, if those seven leave fewer tiles than SMs, heights down to 1 row, with
+   row steps slower the more tiles share an SM. */
 int lbm_batch_set_tile_rows(lbm_batch_h b, int rows);
 /* Set the tiling: output rows and columns per tile and lattice columns per thread (1, or 2
    when the batch's modes include the energy equation and the pseudopotential forces; cols

@@ -156,20 +156,22 @@ double schedule(const lbm_batch *b, const std::vector<const lbm_lattice *> &orde
   return makespan;
 }
 
-// The row steps of the tallest tile of the warp sweep at tile height H (a lattice's rows are
-// divided evenly), which is the launch where every CTA is resident; 0 where they are not.
-int one_wave(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, int H,
-             long long &ntiles) {
+// Time of a launch of the warp sweep at tile height H where every CTA is resident, in row steps
+// of a full SM; 0 where they are not.  The tallest tile (a lattice's rows are divided evenly) is
+// the launch, and a row step takes 0.71, 0.86 and 1 with one, two and three CTAs on the SM, as
+// for the single lattice (lbm_sweep.cu).
+double one_wave(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, int H) {
   long long ctas = 0;
   int tallest = 0;
-  ntiles = 0;
   for (const lbm_lattice *h : order) {
     const int rows = std::min(H, h->ny), chunks = (h->ny + rows - 1) / rows;
     ctas += lbm::sweep_batch_ctas(h->dp, chunks);
-    ntiles += (long long)lbm::sweep_batch_strips(h->dp) * chunks;
     tallest = std::max(tallest, (h->ny + chunks - 1) / chunks);
   }
-  return ctas <= b->sweep_slots ? tallest + lbm::sweep_batch_fill(b->mode.thermal != 0) : 0;
+  if (ctas > b->sweep_slots) return 0.0;
+  const long long per_sm = (ctas + b->sms - 1) / b->sms, occ = b->sweep_slots / b->sms;
+  return (0.57 + 0.43 * (double)per_sm / occ) *
+         (tallest + lbm::sweep_batch_fill(b->mode.thermal != 0));
 }
 
 // Default tile height.  Each candidate of 128 .. 16 rows is scored by the makespan of its
@@ -183,8 +185,18 @@ int one_wave(const lbm_batch *b, const std::vector<const lbm_lattice *> &order, 
 // with 16-bit storage, four: one CTA alone is bound by the latency of its row step, a
 // full SM shares the issue slots), so that a few small lattices spread over the SMs
 // (200 x 50 alone: 1 row, 17.0 against 39.3 us per update with 16; 1024 x 128: 4 rows,
-// 22.8 against 39.6 us).  The figures are the CTA kernel's; the warp sweep is scheduled by
-// the same rule with its own row steps and CTAs.
+// 22.8 against 39.6 us).  The figures are the CTA kernel's.
+//
+// In the warp sweep the heights that make one wave compete by the time of that wave
+// (one_wave): every height up to 24 rows, so that a few small lattices spread over the SMs,
+// and the multiples of four up to 256.  GB300, FP32, us per update at the height chosen, at the
+// fastest of twelve and at 16 rows: 1024 x 128 alone 16.1 (5 rows), 15.6 (3), 28.2; 8 of 200 x 50
+// 14.2 (3), 14.0 (3), 24.8; 24 of them 19.1 (5), 20.2 (3), 25.5; 12 of 512 x 64 22.8 (9), 22.7 (8),
+// 29.0; 48 of 100 x 32 17.0 (3), 16.9 (3), 30.3; 8 uneven ones of 64-464 x 16-80 15.2 (3),
+// 14.3 (2), 28.9.  16 channels of 2.9 M nodes 76.8 at 36 (chosen), 91.9 at 48; 20 of 3.8 M 91.1 at
+// 44 (chosen), 98.0 at 48; 30 of 4.1 M 108.9 at 56 (chosen), 121.4 at 64.  In several waves the
+// schedule does not tell heights close apart (40 channels of 6.3 M nodes 170.4 at 96 rows and
+// 163.5 at 92 in one wave, 178.7 at 40 in two), so those stay the seven.
 int default_rows(const lbm_batch *b, bool sweep) {
   static const int tall[] = {128, 96, 64, 48, 32, 24, 16};
   static const int small[] = {16, 12, 8, 6, 4, 3, 2, 1};
@@ -209,24 +221,18 @@ int default_rows(const lbm_batch *b, bool sweep) {
       best_tiles = n;
     }
   }
-  // In the warp sweep every fourth height from 24 to 256 rows competes too where it makes one
-  // wave: the tallest tile is then the launch (GB300, FP32, us per update: 16 channels of 2.9 M
-  // nodes 91.9 at 48 rows, 76.8 at 36; 30 of 4.1 M 121.4 at 64, 108.9 at 56; 20 channels 98.0 at
-  // 48, 91.1 at 44; FP16 storage 109.9 and 90.6, 140.7 and 127.8).  In several waves the
-  // schedule does not tell heights so close apart (40 channels of 6.3 M nodes 170.4 at 96 rows
-  // and 163.5 at 92 in one wave, 178.7 at 40 in two; 96 channels 432.9 at 64 and 435.2 at 52, both in several).
-  if (sweep)
-    for (int H = 256; H >= 24; H -= 4) {
-      long long n = 0;
-      const int cost = one_wave(b, order, H, n);
-      if (cost > 0 && cost < best_cost) {
+  if (sweep) {
+    for (int H = 256; H >= 1; H -= H > 24 ? 4 : 1) {
+      const double cost = one_wave(b, order, H);
+      if (cost > 0.0 && cost < best_cost) {
         best = H;
         best_cost = cost;
-        best_tiles = n;
       }
     }
+    return best;
+  }
   if (best_tiles >= b->sms) return best;
-  const int occ = std::max(1, std::min(4, (sweep ? b->sweep_slots : b->grid_of[b->cpt]) / b->sms));
+  const int occ = std::max(1, std::min(4, b->grid_of[b->cpt] / b->sms));
   const double *kStep = occ >= 4 ? kStep4 : kStep3;
   best_cost = 0.0;
   for (int H : small) {

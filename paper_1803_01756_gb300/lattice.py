@@ -179,9 +179,11 @@ def _stream_ptr(stream) -> int:
     if stream is None:
         try:
             import torch
-            if torch.cuda.is_initialized():
-                # the current stream's handle without a Stream object
-                return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            if raw is not None and torch.cuda.is_initialized():
+                # the current stream's handle without a Stream object (a private call, which
+                # not every torch has)
+                return raw(torch.cuda.current_device())
             if torch.cuda.is_available():
                 return torch.cuda.current_stream().cuda_stream
         except ImportError:

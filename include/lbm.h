@@ -52,16 +52,17 @@ extern "C" {
 #define LBM_STORAGE_BF16 1   /* stored as BF16 f_i / w_i - rho_ref (FP32 arithmetic) */
 #define LBM_STORAGE_F16 2    /* stored as FP16 f_i / w_i - rho_ref (FP32 arithmetic) */
 
-#define LBM_KERNEL_AUTO 0    /* the library's choice: with the energy equation on, the two-pass
-                                path for lattices of at most 2^18 nodes, else the fused update
-                                by rows of warps, one launch per update, two columns per thread */
+#define LBM_KERNEL_AUTO 0    /* the library's choice, one launch per update, two columns per
+                                thread: on lattices of at most 2^18 nodes streaming, collision
+                                and energy update as phases over tiles (lbm_info gives
+                                LBM_KERNEL_TWOPASS, without the energy equation _FUSED), beyond
+                                the fused update by independent warps (_FUSED) */
 #define LBM_KERNEL_SPLIT 1   /* density/psi, collide, energy: three launches per update */
 #define LBM_KERNEL_FUSED 2   /* one launch per update; the library picks the columns per thread */
 #define LBM_KERNEL_FUSED_1COL 3 /* the fused kernel with one lattice column per thread */
 #define LBM_KERNEL_FUSED_2COL 4 /* the fused kernel with two lattice columns per thread */
-#define LBM_KERNEL_TWOPASS 5 /* streaming and collision (Eqs. 6-15), then the RK4 energy update
-                                (Eqs. 16-18): on lattices of at most 2^18 nodes as the phases
-                                of one launch over tiles, beyond as two launches per update */
+#define LBM_KERNEL_TWOPASS 5 /* two launches per update: streaming and collision (Eqs. 6-15),
+                                then the RK4 energy update (Eqs. 16-18) */
 
 /* Problem parameters, copied by value at lbm_create (the caller keeps ownership). */
 typedef struct lbm_params {
@@ -106,8 +107,8 @@ typedef struct lbm_info {
   size_t device_bytes;        /* device memory held by the handle */
   int kernel;                 /* kernel path in use (LBM_KERNEL_SPLIT, _FUSED or _TWOPASS) */
   int tile_cols, tile_rows;   /* most output columns and rows of one CTA (of one warp, where the
-                                 library's choice sweeps by warps; two-pass path in two
-                                 launches: its first pass; 0 on the split path) */
+                                 library's choice sweeps by warps; two launches per update: the
+                                 first; 0 on the split path) */
   int cols_per_thread;        /* lattice columns each thread works on (1 or 2; 0 on the split
                                  path) */
 } lbm_info_t;

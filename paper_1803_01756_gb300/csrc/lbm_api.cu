@@ -699,23 +699,15 @@ int lbm_create(int nx, int ny, const lbm_params_t *p, lbm_h *out) {
   if (p->x_bc == LBM_X_PRESSURE_INLET)
     h->rho_branch_end = vapour_branch_end(*p, h->Tc, h->Tc * p->T_inlet);
   h->kernel = LBM_KERNEL_SPLIT;
-  // Lattices of at most 2^18 nodes take the tile kernel, where the two-pass path and the
-  // library's choice meet: all rows of a tile at once instead of a pipeline along the rows
-  // (GB300, us per update, two-pass kernels / tile kernel: 200 x 50 9.6 / 3.6, 1600 x 48 13.9 /
-  // 4.3, 1024 x 128 14.7 / 6.7, 777 x 333 18.9 / 11.7, where the warp sweep takes 17.4;
-  // 2048 x 256 28.1 / 21.6, and 21.3 with the warp sweep, which is ahead beyond).
+  // The library's choice for lattices of at most 2^18 nodes is the tile kernel: all rows of a
+  // tile at once instead of a pipeline along the rows (GB300, us per update, two-pass kernels /
+  // tile kernel: 200 x 50 9.6 / 3.6, 1600 x 48 13.9 / 4.3, 1024 x 128 14.7 / 6.7, 777 x 333 18.9 /
+  // 11.7, where the warp sweep takes 17.4; 2048 x 256 28.1 / 21.6, and 21.3 with the warp sweep,
+  // which is ahead beyond).
   const bool small = (long long)nx * ny <= (1LL << 18) && lbm::fused_supported(h->dp);
-  if (small && ((p->kernel == LBM_KERNEL_AUTO) || p->kernel == LBM_KERNEL_TWOPASS)) {
-    int height = 0;
-    // LBM_TWOPASS_TILE="Ha,Hb" sets the rows per CTA to Ha (tuning experiments)
-    if (const char *env = p->kernel == LBM_KERNEL_TWOPASS ? std::getenv("LBM_TWOPASS_TILE") : nullptr) {
-      int Ha = 0, Hb = 0;
-      if (std::sscanf(env, "%d,%d", &Ha, &Hb) == 2 && Ha >= 1 && Hb >= 1) height = Ha;
-    }
-    h->tile = lbm::tile_tiling(h->dp, p->storage, h->device, height);
-    if (h->tile.strips > 0)
-      h->kernel = p->kernel == LBM_KERNEL_TWOPASS || p->thermal ? LBM_KERNEL_TWOPASS
-                                                                : LBM_KERNEL_FUSED;
+  if (small && p->kernel == LBM_KERNEL_AUTO) {
+    h->tile = lbm::tile_tiling(h->dp, p->storage, h->device);
+    if (h->tile.strips > 0) h->kernel = p->thermal ? LBM_KERNEL_TWOPASS : LBM_KERNEL_FUSED;
   }
   if (h->tile.strips > 0) {
     // chosen above

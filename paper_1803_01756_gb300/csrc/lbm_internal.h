@@ -146,8 +146,8 @@ struct TileTiling {
   int width;           // output columns of a strip
   int height;          // most rows of a CTA, swept tile by tile
 };
-// tiling for this device: the library's choice, or `height` rows per CTA when positive
-TileTiling tile_tiling(const DevParams &p, int storage, int device, int height);
+// tiling for this device
+TileTiling tile_tiling(const DevParams &p, int storage, int device);
 int tile_max_rows(bool thermal);
 // sc: the update's scalars in device memory, or nullptr to pass them by value
 cudaError_t launch_tile(const DevParams &p, int storage, const void *gs, void *gout,

@@ -21,17 +21,13 @@ cudaError_t occupancy(const DevParams &p, int storage, int rows, int *occ) {
 
 }  // namespace
 
-TileTiling tile_tiling(const DevParams &p, int storage, int device, int height) {
+TileTiling tile_tiling(const DevParams &p, int storage, int device) {
   TileTiling best{0, 0, 0, 0, 0};
   int sms = 0;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess)
     return best;
   const bool th = p.thermal != 0;
   const int strips = sweep_strips(p.nx, th), most = tile_max_rows(th), fill = 2 * sweep_rows(th);
-  if (height > 0) {
-    best = TileTiling{strips, ceil_div(p.ny, height), rows_of(height, most), sweep_width(th), height};
-    return best.chunks <= 65535 ? best : TileTiling{0, 0, 0, 0, 0};
-  }
   // The height of a CTA's rows with the shortest launch: waves of CTAs (the registers leave
   // one of 20 warps on an SM, and one of 12), each of tiles one after another, and a tile
   // takes 0.70 us and 0.0875 us a warp (GB300, FP32: 200 x 50 with tiles of 2 rows, 12 warps,

@@ -705,7 +705,12 @@ int lbm_create(int nx, int ny, const lbm_params_t *p, lbm_h *out) {
   // 11.7, where the warp sweep takes 17.4; 2048 x 256 28.1 / 21.6, and 21.3 with the warp sweep,
   // which is ahead beyond).
   const bool small = (long long)nx * ny <= (1LL << 18) && lbm::fused_supported(h->dp);
-  if (small && p->kernel == LBM_KERNEL_AUTO) {
+  // LBM_FUSED_TILE and LBM_FUSED_CPT (below) are the CTA sweep's: a lattice of the library's
+  // choice takes that kernel where one of them is set, but for the sizes on which the library
+  // does not choose a sweep with the energy equation
+  const bool tuned = p->kernel == LBM_KERNEL_AUTO && !(small && p->thermal) &&
+                     (std::getenv("LBM_FUSED_TILE") || std::getenv("LBM_FUSED_CPT"));
+  if (small && p->kernel == LBM_KERNEL_AUTO && !tuned) {
     h->tile = lbm::tile_tiling(h->dp, p->storage, h->device);
     if (h->tile.strips > 0) h->kernel = p->thermal ? LBM_KERNEL_TWOPASS : LBM_KERNEL_FUSED;
   }
@@ -726,7 +731,7 @@ int lbm_create(int nx, int ny, const lbm_params_t *p, lbm_h *out) {
       return LBM_ERR_ARG;
     }
     h->kernel = LBM_KERNEL_TWOPASS;
-  } else if (p->kernel == LBM_KERNEL_AUTO && lbm::fused_supported(h->dp) &&
+  } else if (p->kernel == LBM_KERNEL_AUTO && !tuned && lbm::fused_supported(h->dp) &&
              // the library's choice of fused kernel: independent warps (64.6 -> 47.9 us per
              // update on 4096 x 512, 902 -> 561 us on 16384 x 2048; 16-bit storage 70.3 ->
              // 54.0 us)

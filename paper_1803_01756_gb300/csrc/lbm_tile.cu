@@ -34,12 +34,13 @@ TileTiling tile_tiling(const DevParams &p, int storage, int device) {
   // 3.55 us per update, of which 1.8 are the launch and the first loads; 1600 x 48 with 10
   // rows, 20 warps, 4.33; 777 x 333 with 150 CTAs of four such tiles 11.7).
   double best_cost = -1.0;
+  int occ_of[TW + 1] = {};  // resident CTAs per SM by rows of a tile, 0 until asked for
   for (int h = 1; h <= p.ny; h = h < 64 ? h + 1 : h + 16) {
     const int chunks = ceil_div(p.ny, h);
     if (chunks > 65535) continue;
     const int rows = rows_of(h, most), tiles = ceil_div(h, rows);
-    int occ = 0;
-    if (occupancy(p, storage, rows, &occ) != cudaSuccess || occ < 1) return best;
+    int &occ = occ_of[rows];
+    if (occ == 0 && (occupancy(p, storage, rows, &occ) != cudaSuccess || occ < 1)) return best;
     const long long slots = (long long)sms * occ;
     const long long waves = ((long long)strips * chunks + slots - 1) / slots;
     const double cost = (double)waves * tiles * (0.70 + 0.0875 * (rows + fill));

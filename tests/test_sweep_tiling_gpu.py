@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("nx,ny,over,rows", [
     (1000, 300, dict(), 5), (1000, 300, dict(x_bc=0), 5), (520, 510, dict(), 6),
     (1237, 531, dict(), 7), (4096, 512, dict(), 22), (16384, 2048, dict(), 342),
-    (1000, 300, dict(thermal=0), 4),
+    (1000, 300, dict(thermal=0), 4), (2048, 512, dict(), 12),
 ])
 def test_chunk_height_follows_the_size(nx, ny, over, rows):
     torch = pytest.importorskip("torch")

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(SNT, SMIN)
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const int cols = sweep_cols(e.strips), local = b - e.begin;
   const SweepTile t =
-      sweep_tile<sweep_div<YW, XO, ST>()>(e.strips, local % cols, local / cols, warp);
+      sweep_tile<sweep_div<YW, XO, TH, MP, ST>()>(e.strips, local % cols, local / cols, warp);
   if (t.chunk >= e.chunks) return;
   const int Y0 = (int)(((long long)t.chunk * e.p.ny) / e.chunks);
   const int ye = (int)(((long long)(t.chunk + 1) * e.p.ny) / e.chunks);

@@ -29,7 +29,7 @@ __host__ __device__ constexpr int sweep_rows_of_ctas(int strips, int chunks) {
 // same numbers; with one or the other the compiler schedules the row steps differently (GB300,
 // 4096 x 512, us per update, DIV / not: open ends FP32 47.7 / 48.2, FP16 53.5 / 54.0; doubly
 // periodic FP32 54.5 / 66.1, FP16 60.0 / 54.2; walls with periodic x FP32 55.5 / 52.7, 1237 x 531
-// FP16 30.4 / 26.6).
+// FP16 30.4 / 26.6; open ends without the pseudopotential FP32 47.2 / 43.3).
 struct SweepTile {
   int strip, chunk;
 };
@@ -43,9 +43,9 @@ __device__ __forceinline__ SweepTile sweep_tile(int strips, int bx, int by, int 
   const int sh = strips == 1 ? 2 : strips == 2 ? 1 : 0;
   return SweepTile{bx * SW + (warp & ((SW - 1) >> sh)), (by << sh) + (warp >> (2 - sh))};
 }
-template <bool YW, bool XO, class ST>
+template <bool YW, bool XO, bool TH, bool MP, class ST>
 __host__ __device__ constexpr bool sweep_div() {
-  return XO || (!YW && sizeof(typename ST::T) == 4);
+  return (MP || !TH) && (XO || (!YW && sizeof(typename ST::T) == 4));
 }
 // Resident CTAs per SM the registers are sized for: 12 warps with 168 registers a thread.
 // Eight warps with 214 registers let the compiler keep more constants but cover less of the
@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(SNT, SMIN)
   __shared__ float4 rings[SW][TH ? 4 * 3 * 32 : 32];
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
   const SweepTile t =
-      sweep_tile<sweep_div<YW, XO, ST>()>(strips, (int)blockIdx.x, (int)blockIdx.y, warp);
+      sweep_tile<sweep_div<YW, XO, TH, MP, ST>()>(strips, (int)blockIdx.x, (int)blockIdx.y, warp);
   // (a warp beyond the last strip sweeps without a store: returning here is 3 % slower on
   // 1237 x 531)
   if (t.chunk >= chunks) return;

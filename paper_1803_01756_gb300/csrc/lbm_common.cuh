@@ -132,8 +132,8 @@ struct DevParams {
   float rho_out;
 };
 
-// Physics constants of the warp sweep (lbm_sweep.cuh), derived from DevParams by
-// sweep_consts: some with their sign turned or summed.
+// Physics constants of the warp sweep and the tile kernel (lbm_lane.cuh), derived from
+// DevParams by sweep_consts: some with their sign turned or summed.
 struct SweepConsts {
   float rho_ref, b, inv_Tc, xr;
   float sr, nkappa, kappa1r, ps_g, ps_RT, ps_R, ps_phi, ps_B, ps_3, psi_r2, psi_den;

@@ -1,11 +1,12 @@
-// Fused lattice update by independent warps: the sweep shared by the single-lattice kernel
-// (lbm_sweep.cu).
+// Fused lattice update by independent warps: the sweep that the single-lattice kernel
+// (lbm_sweep_launch.cuh) and the batched one (lbm_sweep_batch.cuh) share.
 //
 // A warp owns a strip of 64 lattice columns (two adjacent columns per lane, the first one
-// even) and a chunk of rows, and sweeps the rows upward.  Everything a node needs from
-// other rows stays in the lane's registers, everything it needs from other columns comes
-// from the neighbouring lanes by shuffles, so there is no shared memory and no barrier, and
-// the warps of an SM drift freely past one another.  Per swept row r:
+// even) and a chunk of rows, and sweeps the rows upward.  What a node needs from other rows
+// stays in the lane's registers, but for the values that a node's own RK4 stages share over
+// four row steps: those are in a ring in shared memory that only the lane itself reads (6 KB a
+// warp).  What it needs from other columns comes from the neighbouring lanes by shuffles.  So
+// there is no barrier, and the warps of an SM drift freely past one another.  Per swept row r:
 //   S0 row r   : pull-streaming with boundary rules (Eq. 12), moments, density (Eq. 13),
 //                pseudopotential deviation (Eqs. 10-11)
 //   S1 row r-1 : forces (Eqs. 9, 14, 15), velocity (Eq. 13), MRT collision with Li forcing

@@ -349,7 +349,7 @@ class Lattice:
 
 
 class Batch:
-    """Lattices advanced together, one persistent launch per step (lbm_batch_*).
+    """Lattices advanced together, one launch per step (lbm_batch_*).
 
     The lattices stay owned by the caller and must outlive the batch."""
 

@@ -60,9 +60,9 @@ SM_MAX_MHZ = 2070
 # cycle).  They hold for the kernel sources whose hash is FUSED_COUNTERS_SOURCE (the
 # profiles/ summary of the capture records the same hash); when the built sources hash
 # differently the counters are stale and the bench reports them as null.
-FUSED_F32_4096x512_DRAM_BYTES = 103.403264e6 + 39.863040e6
+FUSED_F32_4096x512_DRAM_BYTES = 103.420928e6 + 40.425216e6
 FUSED_F32_4096x512_WARP_INSTR = 43732808
-FUSED_COUNTERS_SOURCE = "9219133cdaaedea1"
+FUSED_COUNTERS_SOURCE = "813c91cdd4c0e711"
 # the files that determine the fused kernel's machine code
 FUSED_SOURCES = ["paper_1803_01756_gb300/csrc/lbm_common.cuh",
                  "paper_1803_01756_gb300/csrc/lbm_internal.h",
@@ -72,14 +72,49 @@ FUSED_SOURCES = ["paper_1803_01756_gb300/csrc/lbm_common.cuh",
                  "paper_1803_01756_gb300/build.py"]
 
 
-def fused_source_hash() -> str:
-    """First 16 hex digits of the SHA-256 of the fused kernel's source files."""
+# the same counters of one k_sweep launch, the library's choice on that channel
+SWEEP_F32_4096x512_DRAM_BYTES = 121.253376e6 + 43.191296e6
+SWEEP_F32_4096x512_WARP_INSTR = 30859890
+SWEEP_COUNTERS_SOURCE = "fefc0f06e47b0828"
+SWEEP_SOURCES = ["paper_1803_01756_gb300/csrc/lbm_common.cuh",
+                 "paper_1803_01756_gb300/csrc/lbm_internal.h",
+                 "paper_1803_01756_gb300/csrc/lbm_lane.cuh",
+                 "paper_1803_01756_gb300/csrc/lbm_sweep.cuh",
+                 "paper_1803_01756_gb300/csrc/lbm_sweep_launch.cuh",
+                 "paper_1803_01756_gb300/csrc/lbm_sweep.cu",
+                 "paper_1803_01756_gb300/build.py"]
+
+
+def source_hash(files) -> str:
+    """First 16 hex digits of the SHA-256 of the source files."""
     import hashlib
     h = hashlib.sha256()
-    for rel in FUSED_SOURCES:
+    for rel in files:
         with open(os.path.join(ROOT, rel), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
+
+
+def fused_source_hash() -> str:
+    return source_hash(FUSED_SOURCES)
+
+
+def stored_counters(kernel, storage, workload, physics, cols_per_thread):
+    """(DRAM bytes, warp instructions, hash of the built sources, hash of the captured ones) of
+    a launch of the kernel; the first two None where none are stored for the configuration or
+    the sources have changed since."""
+    if kernel == "k_sweep":
+        built, captured = source_hash(SWEEP_SOURCES), SWEEP_COUNTERS_SOURCE
+        counts = (SWEEP_F32_4096x512_DRAM_BYTES, SWEEP_F32_4096x512_WARP_INSTR)
+        stored = True
+    else:
+        built, captured = fused_source_hash(), FUSED_COUNTERS_SOURCE
+        counts = (FUSED_F32_4096x512_DRAM_BYTES, FUSED_F32_4096x512_WARP_INSTR)
+        stored = kernel == "k_fused_step" and cols_per_thread == 1
+    if not (stored and built == captured and storage == "f32" and physics == "full"
+            and workload == "channel_4096x512"):
+        counts = (None, None)
+    return (*counts, built, captured)
 
 
 # --physics: which parts of the update run (the energy equation of Eqs. 16-18 and the
@@ -354,12 +389,10 @@ def our_arm(args, world, rank, local, dist):
     else:
         per_cell = SPLIT_KERNEL_BYTES[top_name]
     traffic = args.traffic
-    src_hash = fused_source_hash()
-    counters_current = src_hash == FUSED_COUNTERS_SOURCE
-    if (traffic is None and top_name == "k_fused_step" and args.storage == "f32"
-            and args.workload == "channel_4096x512" and args.physics == "full"
-            and info["cols_per_thread"] == 1 and counters_current):
-        traffic = FUSED_F32_4096x512_DRAM_BYTES
+    dram, instr, src_hash, counters_hash = stored_counters(
+        top_name, args.storage, args.workload, args.physics, info["cols_per_thread"])
+    if traffic is None:
+        traffic = dram
     bytes_per_launch = per_cell * cells
     avg_us = elapsed_ms * shares[top_name] / top_n * 1e3
     achieved = bytes_per_launch / (avg_us / 1e6) / 1e9
@@ -372,17 +405,17 @@ def our_arm(args, world, rank, local, dist):
                                   f"{args.steps} updates"),
                 "event_bracketed_launch_us": top_ms / top_n * 1e3,
                 "kernel_share": shares, "kernel_source_sha": src_hash,
-                "counters_source_sha": FUSED_COUNTERS_SOURCE}
-    if traffic is not None and args.traffic is None:
+                "counters_source_sha": counters_hash}
+    if instr is not None and args.traffic is None:
         # the same kernel, workload and storage as the ncu counts: its issue roofline
         sms = torch.cuda.get_device_properties(local).multi_processor_count
         mhz = (clocks or {}).get("sm_max_mhz") or SM_MAX_MHZ
         issue_peak = sms * 4 * mhz * 1e6
-        issue = FUSED_F32_4096x512_WARP_INSTR / (avg_us / 1e6)
+        issue = instr / (avg_us / 1e6)
         roofline["issue"] = {
             "achieved": issue / 1e9, "peak": issue_peak / 1e9, "unit": "G warp-instr/s",
             "frac": issue / issue_peak,
-            "instr_per_cell_update": FUSED_F32_4096x512_WARP_INSTR * 32 / cells,
+            "instr_per_cell_update": instr * 32 / cells,
             "peak_source": f"{sms} SMs x 4 schedulers x {mhz:.0f} MHz"}
 
     # ---- end to end through the C ABI with host buffers ----
@@ -435,7 +468,7 @@ def our_arm(args, world, rank, local, dist):
                               f"each ({sum(repeats) / 1e3:.2f} s in all; min "
                               f"{min(repeats) / args.steps * 1e3:.2f}, max "
                               f"{max(repeats) / args.steps * 1e3:.2f} us per update)"),
-                   "kernel": {1: "split", 2: "fused", 5: "twopass"}[info["kernel"]],
+                   "kernel": " + ".join(sorted(per_kernel)),
                    "tile": [info["tile_cols"], info["tile_rows"]],
                    "cols_per_thread": info["cols_per_thread"],
                    "launch": ("16-update CUDA graphs"
@@ -470,15 +503,16 @@ def batch_channels(n: int = 96, seed: int = 3):
 
 
 def batch_arm(args):
-    """MLUPS of one persistent launch per update over the batch mix, against the same
-    lattices advanced one after another with lbm_step."""
+    """MLUPS of the batch mix advanced together on the library's kernel choice, against the
+    same lattices advanced one after another with lbm_step, on the fused kernel and on the
+    library's choice."""
     import torch
     from paper_1803_01756_gb300 import lattice as L
     torch.cuda.set_device(0)
     specs = batch_channels()
     lats = []
     for nx, ny, p, rho0 in specs:
-        lat = L.Lattice(nx, ny, p, kernel=L.KERNEL_FUSED)
+        lat = L.Lattice(nx, ny, p)
         lat.write_fields(rho0)
         lats.append(lat)
     cells = sum(nx * ny for nx, ny, _, _ in specs)
@@ -495,37 +529,33 @@ def batch_arm(args):
     ms = e0.elapsed_time(e1)
     b.close()
     seq_steps = max(1, min(args.steps, 200))
-    for lat in lats:
-        lat.step(2, stream)
-    torch.cuda.synchronize()
-    e0.record(stream)
-    for lat in lats:
-        lat.step(seq_steps, stream)
-    e1.record(stream)
-    torch.cuda.synchronize()
-    seq_ms = e0.elapsed_time(e1)
     status = 0
     for lat in lats:
         status |= lat.status()
         lat.close()
-    # the same, each lattice on the library's own kernel choice (the two-pass path for
-    # lattices of at most 2^18 nodes)
-    auto = []
-    for nx, ny, p, rho0 in specs:
-        lat = L.Lattice(nx, ny, p)
-        lat.write_fields(rho0)
-        lat.step(2, stream)
-        auto.append(lat)
-    torch.cuda.synchronize()
-    e0.record(stream)
-    for lat in auto:
-        lat.step(seq_steps, stream)
-    e1.record(stream)
-    torch.cuda.synchronize()
-    auto_ms = e0.elapsed_time(e1)
-    for lat in auto:
-        status |= lat.status()
-        lat.close()
+
+    def one_after_another(kernel):
+        alone = []
+        for nx, ny, p, rho0 in specs:
+            lat = L.Lattice(nx, ny, p, kernel=kernel)
+            lat.write_fields(rho0)
+            lat.step(2, stream)
+            alone.append(lat)
+        torch.cuda.synchronize()
+        e0.record(stream)
+        for lat in alone:
+            lat.step(seq_steps, stream)
+        e1.record(stream)
+        torch.cuda.synchronize()
+        bits = 0
+        for lat in alone:
+            bits |= lat.status()
+            lat.close()
+        return e0.elapsed_time(e1), bits
+
+    seq_ms, bits = one_after_another(L.KERNEL_FUSED)
+    auto_ms, more = one_after_another(L.KERNEL_AUTO)
+    status |= bits | more
     line = {
         "metric": "lattice updates per second (MLUPS), batched channels", "value":
         cells * args.steps / ms / 1e3, "unit": "MLUPS", "n_gpus": 1, "steps": args.steps,
@@ -535,7 +565,7 @@ def batch_arm(args):
                    "tiles": info["tiles"], "tile_rows": info["tile_rows"], "grid": info["grid"]},
         "sequential_mlups": cells * seq_steps / seq_ms / 1e3,
         "sequential_library_choice_mlups": cells * seq_steps / auto_ms / 1e3,
-        "gpu_launches": args.steps,
+        "gpu_launches": args.steps * -(-len(specs) // 48),  # 48 lattices a launch at most
         "status_bits": status,
     }
     print(json.dumps(line), flush=True)
@@ -595,8 +625,7 @@ def serving_arm(args):
     """jobs/hour and latency of the continuous-batching server, with BF16 population
     storage (the headline) and with FP32 storage (the batching gain alone), against the
     same arrivals solved one at a time in FP32 (first come, first served) on the library's
-    kernel choice for each job (the two-pass path for jobs of at most 2^18 nodes, the fused
-    kernel for larger ones)."""
+    kernel choice for each job."""
     import torch
     from paper_1803_01756_gb300 import lattice as L
     torch.cuda.set_device(0)

@@ -45,7 +45,8 @@ def alone(job, storage=0):
 
 # A job in the mix runs in the batched kernel, alone in the single-lattice kernel; the
 # two compute the same update, so each job's fields must agree within the FP32 parity
-# bound in either storage (measured on GB300: bitwise equal in FP32, BF16 and FP16).
+# bound in either storage (BF16 jobs run on the fused kernel too, FP32 ones on the library's
+# choice; test_serving_kernel_gpu.py compares them with default lattices bit for bit).
 SAME_BOUNDS = {0: {"rho": 1e-5, "u": 1e-5, "T": 1e-5},
                1: {"rho": 1e-5, "u": 1e-5, "T": 1e-5}}
 

@@ -1,7 +1,9 @@
 """The fused update by independent warps (the library's choice of kernel for lattices of more
-than 2^18 nodes, and for every size without the energy equation): parity with the FP64 oracle
+than 2^18 nodes): parity with the FP64 oracle
 over the boundary modes at sizes that end strips, column pairs and row chunks everywhere, and
-the same bits for a node wherever it lies in its strip and chunk.
+the same bits for a node wherever it lies in its strip and chunk.  (The small lattices of
+test_parity_without_the_energy_equation run the tile kernel, which shares the lane's arithmetic;
+test_sweep_modes_gpu.py has the sweep without the energy equation, checked by its name.)
 
 Tolerance: the 1e-5 parity bound of the other update paths (test_parity_gpu.rel_errors); for
 FP16 storage the bounds of the precision tests.

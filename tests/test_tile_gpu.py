@@ -1,8 +1,8 @@
-"""The tile kernel (the two-pass path's phases in one launch, lattices of at most 2^18 nodes):
+"""The tile kernel (the library's choice on lattices of at most 2^18 nodes):
 parity with the FP64 oracle where a CTA sweeps several tiles and at the largest size, and the
-same bits for a node wherever it lies.  The boundary modes, degenerate sizes, row heights,
-16-bit storage and graph replay are covered by the two-pass cases of the parity and precision
-tests.  Tolerance: the 1e-5 parity bound of the other update paths.
+same bits for a node wherever it lies.  The boundary modes, degenerate sizes,
+16-bit storage and graph replay are in test_tile_modes_gpu.py.
+Tolerance: the 1e-5 parity bound of the other update paths.
 """
 import numpy as np
 import pytest

@@ -701,8 +701,8 @@ int lbm_create(int nx, int ny, const lbm_params_t *p, lbm_h *out) {
   h->kernel = LBM_KERNEL_SPLIT;
   // The library's choice for lattices of at most 2^18 nodes is the tile kernel: all rows of a
   // tile at once instead of a pipeline along the rows (GB300, us per update, two-pass kernels /
-  // tile kernel: 200 x 50 9.6 / 3.6, 1600 x 48 13.9 / 4.3, 1024 x 128 14.7 / 6.7, 777 x 333 18.9 /
-  // 11.7, where the warp sweep takes 17.4; 2048 x 256 28.1 / 21.6, and 21.3 with the warp sweep,
+  // tile kernel: 200 x 50 9.6 / 3.5, 1600 x 48 13.9 / 4.5, 1024 x 128 14.7 / 7.4, 777 x 333 18.9 /
+  // 13.9, where the warp sweep takes 17.4; 2048 x 256 28.1 / 21.6, and 21.3 with the warp sweep,
   // which is ahead beyond).
   const bool small = (long long)nx * ny <= (1LL << 18) && lbm::fused_supported(h->dp);
   // LBM_FUSED_TILE and LBM_FUSED_CPT (below) are the CTA sweep's: a lattice of the library's
@@ -732,9 +732,9 @@ int lbm_create(int nx, int ny, const lbm_params_t *p, lbm_h *out) {
     }
     h->kernel = LBM_KERNEL_TWOPASS;
   } else if (p->kernel == LBM_KERNEL_AUTO && !tuned && lbm::fused_supported(h->dp) &&
-             // the library's choice of fused kernel: independent warps (64.6 -> 47.9 us per
-             // update on 4096 x 512, 902 -> 561 us on 16384 x 2048; 16-bit storage 70.3 ->
-             // 54.0 us)
+             // the library's choice of fused kernel: independent warps (64.6 -> 47.8 us per
+             // update on 4096 x 512, 902 -> 560 us on 16384 x 2048; 16-bit storage 70.3 ->
+             // 53.6 us)
              (h->sweep = lbm::sweep_tiling(h->dp, p->storage, h->device)).strips > 0) {
     h->kernel = LBM_KERNEL_FUSED;
   } else if (p->kernel != LBM_KERNEL_SPLIT) {

@@ -31,8 +31,8 @@ TileTiling tile_tiling(const DevParams &p, int storage, int device) {
   // The height of a CTA's rows with the shortest launch: waves of CTAs (the registers leave
   // one of 20 warps on an SM, and one of 12), each of tiles one after another, and a tile
   // takes 0.70 us and 0.0875 us a warp (GB300, FP32: 200 x 50 with tiles of 2 rows, 12 warps,
-  // 3.55 us per update, of which 1.8 are the launch and the first loads; 1600 x 48 with 10
-  // rows, 20 warps, 4.33; 777 x 333 with 150 CTAs of four such tiles 11.7).
+  // 3.54 us per update, of which 1.8 are the launch and the first loads; 1600 x 48 with 10
+  // rows, 20 warps, 4.49; 777 x 333 in several waves of tiles of 9 rows 13.9).
   double best_cost = -1.0;
   int occ_of[TW + 1] = {};  // resident CTAs per SM by rows of a tile, 0 until asked for
   for (int h = 1; h <= p.ny; h = h < 64 ? h + 1 : h + 16) {

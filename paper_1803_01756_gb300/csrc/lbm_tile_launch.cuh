@@ -11,10 +11,10 @@ namespace lbm {
 namespace {
 
 // Most warps of a CTA, for which the registers are sized (96 a thread, no spills): 10 output
-// rows and their 10 halo rows a tile.  28 warps (18 rows, 72 registers, spills) give the same
-// rate on lattices of many tiles (777 x 333: 10.5 against 11.7 us per update) and are slower
-// where there are few (200 x 50: 4.3 against 3.5 us, 1600 x 48: 5.1 against 4.3 us); 14 and
-// 16 warps spend too much of a tile on the halo (777 x 333: 18.1 and 13.8 us).
+// rows and their 10 halo rows a tile.  28 warps (18 rows, 72 registers, spills) are faster on
+// lattices of many tiles (777 x 333: 11.5 against 13.9 us per update, 1024 x 128 6.5 against 7.4)
+// and slower where there are few (200 x 50: 4.9 against 3.5 us, 1600 x 48: 5.1 against 4.5 us);
+// 14 and 16 warps spend too much of a tile on the halo (777 x 333: 23.6 and 18.1 us).
 constexpr int TW = 20;
 
 template <bool YW, bool XO, bool TH, bool MP, class ST>
